@@ -106,7 +106,7 @@ struct ReqDesc {
                                  // 2^sW when s = 0), j = 1..8, each as a packed FP32 pair (tensor path)
     float *nu32;           // [F]
     int *scaleB;           // [F * n_tchunks] power-of-two exponent of each operand tile
-    int *scaleW;           // [1] power-of-two exponent of the weight operand
+    int *scaleW;           // [3] power-of-two exponent of the weight operand; series degree D and halvings s
     float *Bp32;           // [N][F][T] wbar_i A (FP32, SIMT delta form)
     float *dref32;         // [F][T]    reference residual (FP32, SIMT delta form)
     float2 *partials;      // [P][n_part] compensated partial chi^2 (hi, lo)
@@ -176,8 +176,7 @@ struct TcLaunch {
     void *arena;             // operand tile arena (device), 128-byte rows
     int64_t arena_rows;
     unsigned *status;
-    int lean;                // 1: every request has no amplitude regions and Kp equal to the launch's padded
-                             // K; 2: no amplitude regions, Kp of any size; 0: otherwise
+    bool alpha;              // some request has amplitude regions
 };
 // The padded K of a tensor-core launch whose largest request K is kp_max.
 inline int tc_launch_kp(int kp_max) { return kp_max <= 16 ? 16 : kp_max <= 32 ? 32 : 64; }

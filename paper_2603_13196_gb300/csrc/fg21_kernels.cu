@@ -272,7 +272,10 @@ __device__ Fin prep_finalize(const ReqDesc &r, float *sh /* [2 NPF + 2 + 2 nwarp
         r.req_stats[0] = nv;
         r.req_stats[1] = f.x;
         r.req_stats[2] = ma;
-        *r.scaleW = f.sW;
+        const SeriesPlan sp = series_plan((double)f.x);
+        r.scaleW[0] = f.sW;
+        r.scaleW[1] = sp.D;
+        r.scaleW[2] = sp.s;
     }
     __syncthreads();
     return f;

@@ -202,7 +202,7 @@ ReqLayout request_layout(const ReqDesc &r, int precision) {
     L.nu32 = align256(sizeof(float) * r.F);
     L.coef2 = tc ? align256(sizeof(unsigned long long) * 8 * (size_t)r.F) : 0;
     L.scaleB = align256(sizeof(int) * (size_t)r.F * r.n_tchunks);
-    L.scaleW = align256(sizeof(int));
+    L.scaleW = align256(3 * sizeof(int));
     const bool delta = precision == FG21_PREC_FP32_DELTA;
     L.Bp32 = delta ? align256(sizeof(float) * (size_t)r.N * r.F * r.T) : 0;
     L.dref32 = delta ? align256(sizeof(float) * (size_t)r.F * r.T) : 0;
@@ -290,12 +290,8 @@ int prepare_requests(Workspace &ws, std::vector<ReqDesc> &reqs, int precision, P
         L.arena = ws.arena;
         L.arena_rows = row;
         L.status = ws.d_status;
-        bool no_alpha = true, full = true;
-        for (int k = 0; k < n; ++k) {
-            no_alpha = no_alpha && reqs[k].Na == 0;
-            full = full && reqs[k].Kp == tc_launch_kp(kp_max);
-        }
-        L.lean = !no_alpha ? 0 : full ? 1 : 2;
+        L.alpha = false;
+        for (int k = 0; k < n; ++k) L.alpha = L.alpha || reqs[k].Na > 0;
     }
     std::memcpy(ws.pinned, reqs.data(), sizeof(ReqDesc) * n);
     return FG21_OK;

@@ -17,29 +17,51 @@
 //
 // One persistent CTA per SM walks a static list of work items (request, tile
 // of 128 points, group of channels); a stage is one channel (one t-chunk) of
-// the tile.  Warp roles (18 warps):
-//   warps 0-7    weight generators: warp w serves the points of tensor-memory
-//                lane quadrant w%4 and half w/4 of the weight columns; each
-//                thread evaluates its point's weights for the channel in
-//                registers, splits them into hi + mid and writes them straight
-//                into tensor memory (tcgen05.st), where the MMA reads its A
-//                operand;
-//   warps 8-15   epilogue: tcgen05.ld of the accumulator rows of quadrant w%4,
-//                half (w-8)/4 of the t-columns; square-and-sum over t, unscale,
-//                compensated sum over channels, one partial chi2 per (point,
-//                item, half);
-//   warp 16      TMA producer: cp.async.bulk.tensor loads of the channel's
-//                operand tile Bop (prepared per request in global memory);
-//   warp 17      MMA issuer (one elected thread) and tensor-memory owner.
+// the tile.  A CTA has two items in hand at once, one in each of two lanes with
+// warps, rings and accumulators of their own that share nothing but the SM
+// (20 warps; l = lane 0, 1):
+//   warps 4l..4l+3       weight generators: warp w serves the 32 points of
+//                        tensor-memory lane quadrant w%4; each thread evaluates
+//                        its point's whole row of weights for the channel in
+//                        registers, splits them into hi + mid and writes them
+//                        straight into tensor memory (tcgen05.st), where the MMA
+//                        reads its A operand;
+//   warps 8+4l..8+4l+3   epilogue: tcgen05.ld of the accumulator rows of quadrant
+//                        w%4; square-and-sum over t, unscale, compensated sum
+//                        over channels, one partial chi2 per (point, item, half
+//                        of the t-columns);
+//   warp 16+l            TMA producer: cp.async.bulk.tensor loads of the
+//                        channel's operand tile Bop (prepared per request in
+//                        global memory);
+//   warp 18+l            MMA issuer (the first is the tensor-memory owner).
 // Shared memory carries only the operand tiles (the B side), so the tensor
-// cores' shared-memory reads are one operand per MMA.  RING (2-4) stage slots
-// each hold an operand tile in shared memory and an accumulator plus a weight
-// block in tensor memory.  Each slot has two mbarriers: `full` completes when
-// the 8 generator warps have stored the weights, the TMA bytes have landed and
-// the 8 epilogue warps have released the slot's accumulator (17 arrivals +
-// transaction bytes); `done` receives the single tcgen05.commit of the stage's
-// MMAs and tells the producers the slot is free and the epilogue the
-// accumulator is ready.
+// cores' shared-memory reads are one operand per MMA.  A lane's ring (1, 2 or 4
+// stage slots) holds operand tiles in shared memory and weight blocks in tensor
+// memory; its one accumulator is written, read and freed in two halves of the
+// t-columns.  Barriers: `full` of a slot completes when the 4 generator warps
+// have stored the weights and the TMA bytes have landed; `acc_free` of a half
+// when the 4 epilogue warps have read it; `acc_done` and the slot's `done` take
+// the tcgen05.commit after the first and after the second half's MMAs, the
+// latter also telling the producers that the slot is free.
+//
+// What bounds it: instruction issue and latency in the sixteen arithmetic warps
+// (FMA pipe about 58 % busy at 24 regions, 100 bins), so the stages are written
+// to spend few instructions besides the arithmetic and to depend on nothing
+// slow:
+//  - every role runs its loops warp-uniformly, and the elected lane issues MMAs,
+//    commits and copies under a predicate.  Issued from a branch that one lane
+//    takes, a stage's six MMAs cost 677 cycles instead of the tensor pipe's 336;
+//  - a stage is straight-line code for its number of region chunks (generators)
+//    and column blocks (epilogue).  With loops over them inside the stage, the
+//    epilogue alone took 1,580 cycles a stage;
+//  - whole rows per warp and one item per lane, rather than two warps on halves
+//    of each row, so that the waits, arrivals and sums of a stage are paid once;
+//  - waits test the barrier before the suspending try_wait, which takes about
+//    125 cycles even when the phase is complete.
+// 16384 points, 24 regions, 301 channels, 100 bins: 97 us (prior draws) and 89 us
+// (near the posterior), from 162 and 158 us with one item in hand, half rows and
+// single-lane issue; 3001 points, 41 regions, 211 channels, 217 bins: 53 us from
+// 71 us.
 // Every wait is bounded (a few seconds of %globaltimer); on expiry the kernel
 // sets a status bit, the roles stop, in-flight MMAs are drained with bounded
 // waits and tensor memory is released before the CTA exits.
@@ -58,11 +80,12 @@ namespace fg21 {
 
 namespace {
 
-constexpr int NUM_THREADS = 576;
-constexpr int MAX_RING = 4;       // stage slots (the launch picks 2-4 by tensor-memory room)
-constexpr int FULL_ARRIVALS = 17; // 8 generator warps + 1 TMA producer + 8 epilogue warps
-constexpr int WARP_TMA = 16, WARP_MMA = 17;
-constexpr int EPI_NB = 4;         // accumulator blocks an epilogue warp loads per wait
+constexpr int NUM_THREADS = 640;  // 20 warps: five share a scheduler's 16,384 registers, so 96 a thread
+constexpr int LANES = 2;          // work items a CTA has in hand at once
+constexpr int MAX_RING = 4;       // stage slots of a lane (the launch picks by tensor- and shared-memory room)
+constexpr int FULL_ARRIVALS = 5;  // a lane's 4 generator warps + its TMA producer
+constexpr int WARP_EPI = 8, WARP_TMA = 16, WARP_MMA = 18;
+constexpr int EPI_NB = 4;         // accumulator blocks whose squares one set of chains sums
 // TMA boxes are 64 x box_rows 16-bit values (128-byte rows); box_rows divides
 // every request's tile height (a multiple of 8, at most 256)
 constexpr uint64_t WAIT_LIMIT_NS = 4000000000ull;
@@ -70,11 +93,14 @@ constexpr uint64_t WAIT_LIMIT_NS = 4000000000ull;
 // until the phase completes) instead of re-polling, leaving issue slots to the
 // warps that compute
 constexpr uint32_t TRY_WAIT_HINT_NS = 10000000u;
+constexpr int WAIT_TRIES = 32;
 
 struct __align__(8) Barriers {
-    uint64_t full[MAX_RING];
-    uint64_t done[MAX_RING];
-    uint64_t drain;
+    uint64_t full[LANES * MAX_RING];
+    uint64_t done[LANES * MAX_RING];
+    uint64_t acc_done[LANES];        // first half of the accumulator written
+    uint64_t acc_free[LANES * 2];    // each half of the accumulator read
+    uint64_t drain[LANES];
     uint32_t tmem_base;
     volatile uint32_t abort_flag;
 };
@@ -103,10 +129,13 @@ __device__ __forceinline__ void mbar_arrive_warp(uint64_t *bar) {
         "@p mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];\n\t}" ::"r"(smem_u32(bar))
         : "memory");
 }
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.release.cta.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
-                 "r"(bytes)
-                 : "memory");
+__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t bytes, uint32_t elected) {
+    asm volatile(
+        "{\n\t.reg .pred e;\n\t"
+        "setp.ne.b32 e, %2, 0;\n\t"
+        "@e mbarrier.arrive.expect_tx.release.cta.shared::cta.b64 _, [%0], %1;\n\t}" ::"r"(smem_u32(bar)),
+        "r"(bytes), "r"(elected)
+        : "memory");
 }
 __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
     uint32_t ok;
@@ -116,6 +145,26 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(ok)
         : "r"(smem_u32(bar)), "r"(parity), "r"(TRY_WAIT_HINT_NS)
+        : "memory");
+    return ok != 0;
+}
+// Up to WAIT_TRIES tries: a waiting warp spends three instructions per try, and
+// looks at the timer and the abort flag only between such runs.
+__device__ __forceinline__ bool mbar_try_waits(uint64_t *bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t.reg .u32 n;\n\t"
+        "mov.u32 n, 0;\n\t"
+        "FG21_TRY:\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+        "@p bra FG21_DONE;\n\t"
+        "add.u32 n, n, 1;\n\t"
+        "setp.lt.u32 q, n, %4;\n\t"
+        "@q bra FG21_TRY;\n\t"
+        "FG21_DONE:\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity), "r"(TRY_WAIT_HINT_NS), "n"(WAIT_TRIES)
         : "memory");
     return ok != 0;
 }
@@ -131,15 +180,19 @@ __device__ __forceinline__ bool mbar_test(uint64_t *bar, uint32_t parity) {
         : "memory");
     return ok != 0;
 }
-// Bounded wait: true when the phase completed; false on timeout or abort.
+// Bounded wait of a converged warp: true when the phase completed; false on
+// timeout or abort.  Votes make the outcome the same in every lane (and the
+// branches on it warp-uniform).
 __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, Barriers *S, unsigned *status,
                                           unsigned code, uint64_t limit_ns = WAIT_LIMIT_NS) {
-    if (mbar_try_wait(bar, parity)) return true;
+    // (a try_wait takes about 125 cycles even on a phase that is complete)
+    if (__all_sync(0xffffffffu, mbar_test(bar, parity))) return true;
+    if (__all_sync(0xffffffffu, mbar_try_waits(bar, parity))) return true;
     const uint64_t t0 = globaltimer();
     while (true) {
-        if (mbar_try_wait(bar, parity)) return true;
-        if (S->abort_flag) return false;
-        if (globaltimer() - t0 > limit_ns) {
+        if (__all_sync(0xffffffffu, mbar_try_waits(bar, parity))) return true;
+        if (__any_sync(0xffffffffu, S->abort_flag != 0)) return false;
+        if (__any_sync(0xffffffffu, globaltimer() - t0 > limit_ns)) {
             atomicOr(status, code);
             S->abort_flag = 1;
             return false;
@@ -152,11 +205,14 @@ __device__ __forceinline__ void tc_fence_before() {
 __device__ __forceinline__ void tc_fence_after() {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
-__device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, int x, int y, uint64_t *bar) {
+__device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, int x, int y, uint64_t *bar,
+                                            uint32_t elected) {
     asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
+        "{\n\t.reg .pred e;\n\t"
+        "setp.ne.b32 e, %5, 0;\n\t"
+        "@e cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n\t}" ::"r"(
             smem_u32(dst)),
-        "l"((uint64_t)map), "r"(x), "r"(y), "r"(smem_u32(bar))
+        "l"((uint64_t)map), "r"(x), "r"(y), "r"(smem_u32(bar)), "r"(elected)
         : "memory");
 }
 // Shared-memory matrix descriptor, K-major, no swizzle: core matrices of 8 rows
@@ -176,36 +232,64 @@ __device__ __forceinline__ uint32_t instr_desc(int M, int N, bool bf16) {
     const uint32_t fmt = bf16 ? 1u : 0u;
     return (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
-// D (+)= A B with A in tensor memory (128 lanes = rows, K packed two 16-bit
-// values per 32-bit column) and B in shared memory.
-__device__ __forceinline__ void mma_f16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b, uint32_t idesc,
-                                           uint32_t accum) {
+// True in one lane of the (converged) warp.
+__device__ __forceinline__ uint32_t elect_one() {
+    uint32_t e;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(e));
+    return e;
+}
+// D (+)= A B with A in tensor memory (128 lanes = rows, K packed two 16-bit
+// values per 32-bit column) and B in shared memory.  Run by the whole converged
+// warp and issued by its elected lane under a predicate: from a branch that only
+// one lane takes, each tcgen05.mma costs about 107 cycles to issue (677 cycles
+// for a stage's six, whatever N); issued this way the six take the 336 cycles
+// the tensor pipe needs for them at N = 112 (105 at N = 16, 192 at N = 64), with
+// the other warps' FMAs and tensor-memory traffic running or not.
+__device__ __forceinline__ void mma_f16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b, uint32_t idesc,
+                                           uint32_t accum, uint32_t elected) {
+    asm volatile(
+        "{\n\t.reg .pred p, e;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "r"(a_tmem), "l"(b), "r"(idesc), "r"(accum)
+        "setp.ne.b32 e, %5, 0;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "r"(a_tmem), "l"(b), "r"(idesc), "r"(accum), "r"(elected)
         : "memory");
 }
-__device__ __forceinline__ void mma_commit(uint64_t *bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-                 : "memory");
-}
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float *v) {
-    uint32_t r[16];
+__device__ __forceinline__ void mma_commit(uint64_t *bar, uint32_t elected) {
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
-#pragma unroll
-    for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
+        "{\n\t.reg .pred e;\n\t"
+        "setp.ne.b32 e, %1, 0;\n\t"
+        "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(smem_u32(bar)),
+        "r"(elected)
+        : "memory");
 }
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t *v) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {"
+                 "%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+                 : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t *v) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {"
+                 "%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+                 : "r"(taddr));
+}
+// Waits for this thread's tensor-memory loads.
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 // This thread's lane, N consecutive 32-bit columns from taddr.
 __device__ __forceinline__ void tmem_st4(uint32_t taddr, const uint32_t *v) {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};" ::"r"(taddr), "r"(v[0]), "r"(v[1]),
                  "r"(v[2]), "r"(v[3])
+                 : "memory");
+}
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t *v) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "r"(v[0]),
+                 "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
                  : "memory");
 }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
@@ -223,6 +307,11 @@ __device__ __forceinline__ void kahan_add_dev(float &s, float &c, float x) {
 }
 
 // ---------------------------------------------------------- work items
+// A value that is the same in every lane of the (converged) warp, told to the
+// compiler as such: loop bounds and slots made of it stay in uniform registers
+// and its branches are warp-uniform.
+__device__ __forceinline__ int uni(int v) { return __shfl_sync(0xffffffffu, v, 0); }
+
 struct Item {
     int req, tile, g, f0, f1;
 };
@@ -230,19 +319,22 @@ __device__ __forceinline__ int find_req(const ReqDesc *__restrict__ reqs, int n,
     int lo = 0, hi = n - 1;
     while (lo < hi) {
         int mid = (lo + hi + 1) >> 1;
-        if (reqs[mid].item_begin <= item) lo = mid; else hi = mid - 1;
+        if (uni(reqs[mid].item_begin <= item)) lo = mid; else hi = mid - 1;
     }
     return lo;
 }
+// Called by a whole converged warp.
 __device__ __forceinline__ Item decode_item(const ReqDesc *__restrict__ reqs, int n, int64_t item) {
     Item it;
     it.req = find_req(reqs, n, item);
     const ReqDesc &r = reqs[it.req];
     const int64_t lid = item - r.item_begin;
-    it.tile = (int)(lid / r.G);
-    it.g = (int)(lid % r.G);
-    it.f0 = it.g * r.ch_per_group;
-    it.f1 = min(r.F, it.f0 + r.ch_per_group);
+    const int tile = (lid >> 32) == 0 ? (int)((uint32_t)lid / (uint32_t)r.G) : (int)(lid / r.G);
+    it.tile = uni(tile);
+    it.g = uni((int)(lid - (int64_t)tile * r.G));
+    const int f0 = it.g * r.ch_per_group;
+    it.f0 = uni(f0);
+    it.f1 = uni(min(r.F, f0 + r.ch_per_group));
     return it;
 }
 
@@ -311,104 +403,23 @@ __device__ __forceinline__ uint32_t pack2(float a, float b) {
         return *reinterpret_cast<uint32_t *>(&h);
     }
 }
-template <bool BF16>
-__device__ __forceinline__ float2 unpack2(uint32_t u) {
-    if (BF16) {
-        __nv_bfloat162 h = *reinterpret_cast<__nv_bfloat162 *>(&u);
-        return __bfloat1622float2(h);
-    } else {
-        __half2 h = *reinterpret_cast<__half2 *>(&u);
-        return __half22float2(h);
-    }
-}
-// split a pair into hi (rounded) and mid (rounded remainder)
+// split a pair into hi (rounded) and mid (rounded remainder); the remainder
+// a - hi by one mixed-precision FMA per value, exact
 template <bool BF16>
 __device__ __forceinline__ void split2(float a, float b, uint32_t &hi, uint32_t &mid) {
     hi = pack2<BF16>(a, b);
-    const float2 h = unpack2<BF16>(hi);
     float ra, rb;
-    upk2(sub2(pk2(a, b), pk2(h.x, h.y)), ra, rb);
+    if (BF16)
+        asm("{\n\t.reg .b16 l, h, m;\n\tmov.b32 {l, h}, %2;\n\tmov.b16 m, 0xBF80;\n\t"
+            "fma.rn.f32.bf16 %0, l, m, %3;\n\tfma.rn.f32.bf16 %1, h, m, %4;\n\t}"
+            : "=f"(ra), "=f"(rb)
+            : "r"(hi), "f"(a), "f"(b));
+    else
+        asm("{\n\t.reg .b16 l, h, m;\n\tmov.b32 {l, h}, %2;\n\tmov.b16 m, 0xBC00;\n\t"
+            "fma.rn.f32.f16 %0, l, m, %3;\n\tfma.rn.f32.f16 %1, h, m, %4;\n\t}"
+            : "=f"(ra), "=f"(rb)
+            : "r"(hi), "f"(a), "f"(b));
     mid = pack2<BF16>(ra, rb);
-}
-
-// One channel's weights of this thread's point for its half of the request's
-// Kr columns (nph = Kr/4 pairs, at most NPHMAX; FULL: nph = NPHMAX), written
-// to tensor memory: hi at columns t_hi.., mid at t_mid.. (one 32-bit column
-// per pair: the lower K index in the low half).  Pair i holds deviations d2[i]
-// (zero beyond N -> zero weight); on the last half the final pair is
-// (trough, -1) instead (columns Kr-2, Kr-1).  A chunk whose pairs all lie
-// beyond N (pair index >= nz) is stored as zeros without evaluation.  The
-// Horner chains of a chunk of CH pairs advance together.
-// ALPHA (amplitude regions): the series runs on y = d nL + g with g =
-// ln(alpha / abar) of each component (pairs at gp[i * 128]) and the channel's
-// nL in nL2; e2 then holds the constant coefficients 2^(-s j) / j!.  DF: the
-// series degree fixed at compile time (3, 5 or 8; 0 = the request's sp.D at
-// run time); the lean kernel dispatches on it once per work item.
-template <int NPHMAX, bool BF16, bool FULL, bool ALPHA, int DF = 0>
-__device__ __forceinline__ void gen_half(uint32_t t_hi, uint32_t t_mid, const uint64_t *d2,
-                                         const float2 *__restrict__ lop, const uint64_t *e2, SeriesPlan sp,
-                                         uint64_t sW2, int nph_rt, int nz, bool last, float s21, float sW,
-                                         const float2 *__restrict__ gp, uint64_t nL2) {
-    constexpr int CH = 4;
-    const int nph = FULL ? NPHMAX : nph_rt;
-#pragma unroll
-    for (int c0 = 0; c0 < NPHMAX; c0 += CH) {
-        if (!FULL && c0 >= nph) break;
-        uint64_t w[CH];
-        if (c0 < nz) {
-            const uint64_t *x2 = d2 + c0;
-            uint64_t y2[CH];
-            if (ALPHA) {
-                // nph is a multiple of CH, so every pair of a chunk below nz is below nph
-#pragma unroll
-                for (int i = 0; i < CH; ++i) {
-                    const float2 g = __ldg(gp + (size_t)(c0 + i) * 128);
-                    y2[i] = fma2(d2[c0 + i], nL2, pk2(g.x, g.y));
-                }
-                x2 = y2;
-            }
-            if (DF == 3 || (DF == 0 && sp.D == 3)) {
-                // short series (a batch spread below ~0.007 in beta, as near a
-                // posterior): the deviations' low parts enter the weights
-                uint64_t l2[CH];
-#pragma unroll
-                for (int i = 0; i < CH; ++i) {
-                    const float2 v = ALPHA ? make_float2(0.0f, 0.0f) : __ldg(lop + (size_t)(c0 + i) * 128);
-                    l2[i] = pk2(v.x, v.y);
-                }
-                em1_series2<3, CH, !ALPHA>(w, x2, e2, l2);
-            } else if (DF == 5 || (DF == 0 && sp.D == 5)) {
-                em1_series2<5, CH, false>(w, x2, e2, nullptr);
-            } else {
-                em1_series2<8, CH, false>(w, x2, e2, nullptr);
-            }
-            if (DF != 3 && DF != 5 && sp.s > 0) {
-                const uint64_t two2 = pk2(2.0f, 2.0f);
-                for (int q = 0; q < sp.s; ++q)
-#pragma unroll
-                    for (int i = 0; i < CH; ++i) w[i] = mul2(w[i], add2(w[i], two2));
-#pragma unroll
-                for (int i = 0; i < CH; ++i) w[i] = mul2(w[i], sW2);
-            }
-        } else {
-#pragma unroll
-            for (int i = 0; i < CH; ++i) w[i] = 0;
-        }
-        uint32_t H[CH], M[CH];
-#pragma unroll
-        for (int i = 0; i < CH; ++i) {
-            float a, b;
-            upk2(w[i], a, b);
-            const bool tr = FULL ? (c0 + i == NPHMAX - 1) : (c0 + i == nph - 1);
-            if (last && tr) {
-                a = s21;
-                b = -sW;
-            }
-            split2<BF16>(a, b, H[i], M[i]);
-        }
-        tmem_st4(t_hi + c0, H);
-        tmem_st4(t_mid + c0, M);
-    }
 }
 
 struct Params {
@@ -416,260 +427,377 @@ struct Params {
     int n_reqs;
     int64_t n_items;
     int b_stage_bytes;     // bytes of one operand-tile stage
-    int acc_cols;          // tensor-memory columns of one accumulator slot
-    int ring;              // stage slots (2..MAX_RING)
+    int acc_cols;          // tensor-memory columns of a lane's accumulator
+    int ring_log2;         // a lane's stage slots (operand tile, weight block, barriers): 1, 2 or 4
     uint32_t tmem_cols;    // allocated tensor-memory columns
     unsigned *status;
     float *resid;          // validation mode: residuals [P][F][T] of request 0, else null
     int box_rows;          // rows per TMA box
 };
 
-// Stage counter of a role: slot = stage mod ring, phase parity flips each lap.
-struct Ring {
-    uint32_t slot = 0, ph = 0;
-    __device__ __forceinline__ void next(int ring) {
-        if (++slot == (uint32_t)ring) {
-            slot = 0;
-            ph ^= 1u;
-        }
-    }
-};
+// Slots of a lane's stage k: both rings are powers of two, so a role keeps one
+// counter and masks it (phase parity flips each lap).
+__device__ __forceinline__ uint32_t slot_of(uint32_t k, int ring_log2) { return k & ((1u << ring_log2) - 1u); }
+__device__ __forceinline__ uint32_t phase_of(uint32_t k, int ring_log2) { return (k >> ring_log2) & 1u; }
+
+// A CTA's items: lane l takes items blockIdx.x + gridDim.x (l + LANES j), j = 0, 1, ..
+__device__ __forceinline__ int64_t first_item(int lane_id) { return blockIdx.x + (int64_t)gridDim.x * lane_id; }
+__device__ __forceinline__ int64_t item_step() { return (int64_t)gridDim.x * LANES; }
 
 // ------------------------------------------------------------ generators
-// Generator state of one item: this thread's deviations for its half of the
-// columns, and the request constants.
-template <int NPHMAX>
-struct GenItem {
-    uint64_t d2[NPHMAX];
-    const float2 *lop;     // this thread's first low-part pair of its half (spectral-index-only models)
-    float a21, nu21, inv2s2, sW;
-    int Kr, nz;            // nz: pairs of this half from index nz on carry no region
-    SeriesPlan sp;
-    const float2 *gp;      // amplitude regions: this thread's ln(alpha/abar) pairs of its half, else null
-};
-template <int NPHMAX>
-__device__ __forceinline__ void gen_item_load(GenItem<NPHMAX> &g, const ReqDesc &r, const Item &it, int half,
-                                              int m) {
-    const int Kr = r.Kp, nph = Kr / 4;
+// The weights of one item's stages by one warp (32 points).
+// Per stage: wait until the weight slot is free (the MMAs of stage - ring are
+// done), evaluate the series (the Horner chains of up to 8 region pairs advance
+// together), split and store to tensor memory (hi at columns 0 .. Kr/2-1 of the
+// slot's weight block, mid after them; one 32-bit column per pair, the lower K
+// index in the low half), then one arrival on full[slot].  The last pair of the
+// row is (trough, -1); pairs between the regions and it are zeros.  Returns
+// false on a wait timeout.
+//
+// KR, NEV: the request's K and its chunks of 4 pairs that hold regions, ceil(N /
+// 8), fixed at compile time so that a stage is straight-line code (a stage in a
+// loop over chunks spends more issue slots on control than on the series); KR =
+// 0 takes both at run time, for the forms that are not worth their own code.
+// ALPHA (amplitude regions): the series runs on y = d nL + g with g = ln(alpha
+// / abar) of each component; the coefficients 2^(-s j) / j! are then the same
+// for every channel.  DF: the series degree (3, 5 or 8).  With the short series
+// (D = 3: a batch spread below ~0.007 in beta, as near a posterior) the
+// deviations' low parts enter the weights.
+template <int KP, bool BF16, int KR, int NEV, bool ALPHA, int DF>
+__device__ __forceinline__ bool gen_item(const Params &prm, Barriers *S, uint32_t &stage, uint32_t slot0, const ReqDesc &r, const Item &it,
+                                         SeriesPlan sp, uint32_t w_lane, int m) {
+    constexpr bool FIXED = KR > 0;
+    constexpr int UNITS = (FIXED ? KR : KP) / 16;          // K steps of the row: 8 pairs each
+    constexpr int NP = FIXED ? NEV * 4 : KP / 2;           // pairs that may hold regions
+    constexpr bool LO = DF == 3 && !ALPHA;
+    constexpr bool X2 = LO || ALPHA;                       // a second operand per pair: the low part, or g
+    constexpr bool X2_REGS = X2 && KP <= 32;               // ... kept in registers
+    const int Kr = FIXED ? KR : uni(r.Kp), nch = uni(r.n_tchunks);
+    const int nev = FIXED ? NEV : uni((r.N + 7) / 8);
     const float *__restrict__ pts = r.pts32 + (size_t)it.tile * r.pts_rows * 128 + m;
-    // this half's pairs [half*nph, half*nph + nph): regions 2*pair, 2*pair+1 (zero beyond N)
+    uint64_t d2[NP];
 #pragma unroll
-    for (int i = 0; i < NPHMAX; ++i) {
-        const int k = 2 * (half * nph + i);
-        const float a = (i < nph && k < Kr - 2) ? pts[(size_t)k * 128] : 0.0f;
-        const float b = (i < nph && k + 1 < Kr - 2) ? pts[(size_t)(k + 1) * 128] : 0.0f;
-        g.d2[i] = pk2(a, b);
+    for (int i = 0; i < NP; ++i) {
+        const bool in = 2 * i < Kr - 2;
+        d2[i] = pk2(in ? pts[(size_t)(2 * i) * 128] : 0.0f, in ? pts[(size_t)(2 * i + 1) * 128] : 0.0f);
     }
-    // low parts: pair-interleaved rows after the other operands (pairs beyond N hold zeros)
-    g.lop = reinterpret_cast<const float2 *>(pts - m + (size_t)(Kr + 4 + (r.Na ? Kr : 0)) * 128) +
-            (size_t)half * nph * 128 + m;
-    g.a21 = half ? pts[(size_t)(Kr - 2) * 128] : 0.0f;
-    g.nu21 = half ? pts[(size_t)(Kr - 1) * 128] : 0.0f;
-    g.inv2s2 = half ? pts[(size_t)Kr * 128] : 0.0f;
-    g.sW = exp2i(*r.scaleW);
-    g.sp = series_plan(r.req_stats[1]);
-    g.Kr = Kr;
-    g.nz = min(nph, max(0, (r.N + 1) / 2 - half * nph));
-    g.gp = r.Na ? reinterpret_cast<const float2 *>(pts - m + (size_t)(Kr + 4) * 128) + (size_t)half * nph * 128 + m
-                : nullptr;
-}
-
-// The weights of every stage of one item by one generator warp (FULL: the
-// request's Kr equals the kernel's KP).  Per stage: wait until the weight slot
-// is free (the MMAs of stage - ring are done), evaluate and store the weights,
-// then one arrival on full[slot].  Returns false on a wait timeout.
-template <int KP, bool BF16, bool FULL, bool ALPHA, int DF = 0>
-__device__ __forceinline__ bool gen_item(const Params &prm, Barriers *S, Ring &rg, const ReqDesc &r, const Item &it,
-                                         const GenItem<KP / 4> &gi, uint32_t w_lane, int half) {
-    constexpr int NPHMAX = KP / 4;
-    const int lane = threadIdx.x & 31, nch = r.n_tchunks;
-    const int nph = gi.Kr / 4;
-    const float *__restrict__ nLp = r.nL32;
+    // pair-interleaved rows after the point operands: the components' g, or (no
+    // amplitude regions) the deviations' low parts
+    const float2 *__restrict__ pair2 = reinterpret_cast<const float2 *>(pts - m + (size_t)(Kr + 4) * 128) + m;
+    uint64_t x2[X2_REGS ? NP : 1];
+    if (X2_REGS) {
+#pragma unroll
+        for (int i = 0; i < NP; ++i) {
+            const float2 v = 2 * i < Kr ? __ldg(pair2 + (size_t)i * 128) : make_float2(0.0f, 0.0f);
+            x2[i] = pk2(v.x, v.y);
+        }
+    }
+    const float sW = exp2i(*r.scaleW);
+    const float a21 = sW * pts[(size_t)(Kr - 2) * 128], nu21 = pts[(size_t)(Kr - 1) * 128];
+    const float inv2s2 = pts[(size_t)Kr * 128];
     const float *__restrict__ nup = r.nu32;
-    const float ys = exp2i(-gi.sp.s);
-    const uint64_t sW2 = pk2(gi.sW, gi.sW);
-    float nL_n = __ldg(nLp + it.f0), nu_n = __ldg(nup + it.f0);
+    const float *__restrict__ nLp = r.nL32;
+    const unsigned long long *__restrict__ coef = r.coef2;
+    uint64_t e2[DF + 1];
+    e2[0] = 0;
+    if (ALPHA) {
+        const float ys = exp2i(-sp.s);
+        float pw = sp.s ? 1.0f : sW, fact = 1.0f;
+#pragma unroll
+        for (int j = 1; j <= DF; ++j) {
+            pw *= ys;
+            fact *= (float)j;
+            const float e = pw * (1.0f / fact);
+            e2[j] = pk2(e, e);
+        }
+    }
     for (int f = it.f0; f < it.f1; ++f) {
-        const float nL = nL_n, nuf = nu_n;
-        const int fn = min(f + 1, it.f1 - 1);            // next channel's constants, one ahead
-        nL_n = __ldg(nLp + fn);
-        nu_n = __ldg(nup + fn);
-        // e_j = (nL / 2^s)^j / j! (ALPHA: 2^(-s j) / j!, the series being in y), times 2^sW when s = 0
-        uint64_t e2[9];
-        e2[0] = 0;
+        const float dnu = __ldg(nup + f) - nu21;
+        uint64_t nL2 = 0;
         if (ALPHA) {
-            // constant coefficients 2^(-s j) / j! (the series runs in y)
-            float pw = gi.sp.s ? 1.0f : gi.sW, fact = 1.0f;
-#pragma unroll
-            for (int j = 1; j < 9; ++j) {
-                pw *= ys;
-                fact *= (float)j;
-                const float e = pw * (1.0f / fact);
-                e2[j] = pk2(e, e);
-            }
+            const float nL = __ldg(nLp + f);
+            nL2 = pk2(nL, nL);
         } else {
-            // the channel's coefficients, written by prep as packed pairs
-            const ulonglong2 *cf = reinterpret_cast<const ulonglong2 *>(r.coef2 + (size_t)f * 8);
+            // the channel's coefficients e_j = (nL / 2^s)^j / j! (times 2^sW when s = 0), packed pairs
+            const ulonglong2 *cf = reinterpret_cast<const ulonglong2 *>(coef + (size_t)f * 8);
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
+            for (int j = 0; 2 * j < DF; ++j) {
                 const ulonglong2 v = __ldg(cf + j);
                 e2[2 * j + 1] = v.x;
-                e2[2 * j + 2] = v.y;
+                if (2 * j + 2 <= DF) e2[2 * j + 2] = v.y;
             }
         }
-        float s21 = 0.0f;
-        if (half) {
-            const float dnu = nuf - gi.nu21;
-            s21 = gi.sW * gi.a21 * __expf(-dnu * dnu * gi.inv2s2);
-        }
+        const float s21 = a21 * __expf(-dnu * dnu * inv2s2);
         for (int c = 0; c < nch; ++c) {
-            if (!mbar_wait(&S->done[rg.slot], rg.ph ^ 1, S, prm.status, STATUS_TIMEOUT_GEN)) return false;
-            tc_fence_after();
-            const uint32_t wb = w_lane + rg.slot * KP;
-            if (FULL)
-                gen_half<NPHMAX, BF16, true, ALPHA, DF>(wb + half * NPHMAX, wb + KP / 2 + half * NPHMAX, gi.d2, gi.lop,
-                                                    e2, gi.sp, sW2, NPHMAX, gi.nz, half != 0, s21, gi.sW, gi.gp,
-                                                    pk2(nL, nL));
-            else
-                gen_half<NPHMAX, BF16, false, ALPHA, DF>(wb + half * nph, wb + gi.Kr / 2 + half * nph, gi.d2, gi.lop,
-                                                     e2, gi.sp, sW2, nph, gi.nz, half != 0, s21, gi.sW, gi.gp,
-                                                     pk2(nL, nL));
-            tmem_st_wait();
-            tc_fence_before();
-            __syncwarp();
-            mbar_arrive_warp(&S->full[rg.slot]);
-            rg.next(prm.ring);
+        const uint32_t slot = slot0 + slot_of(stage, prm.ring_log2);
+        if (!mbar_wait(&S->done[slot], phase_of(stage, prm.ring_log2) ^ 1u, S, prm.status, STATUS_TIMEOUT_GEN))
+            return false;
+        tc_fence_after();
+        const uint32_t t_hi = w_lane + slot * KP, t_mid = t_hi + Kr / 2;
+#pragma unroll
+        for (int u = 0; u < UNITS; ++u) {
+            if (!FIXED && 16 * u >= Kr) break;
+            uint32_t H[8], M[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) H[i] = M[i] = 0;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                constexpr int CH = 4;
+                const int q = 2 * u + h;                   // chunk of 4 pairs
+                if (FIXED ? q < NEV : q < nev) {
+                    uint64_t w[CH], y2[CH], l2[CH];
+#pragma unroll
+                    for (int i = 0; i < CH; ++i) {
+                        y2[i] = d2[q * CH + i];
+                        l2[i] = 0;
+                        if (X2_REGS) {
+                            l2[i] = x2[q * CH + i];
+                        } else if (X2) {
+                            const float2 v = __ldg(pair2 + (size_t)(q * CH + i) * 128);
+                            l2[i] = pk2(v.x, v.y);
+                        }
+                        if (ALPHA) y2[i] = fma2(y2[i], nL2, l2[i]);
+                    }
+                    em1_series2<DF, CH, LO>(w, y2, e2, l2);
+                    if (DF == 8 && !FIXED && sp.s > 0) {
+                        const uint64_t two2 = pk2(2.0f, 2.0f), sW2 = pk2(sW, sW);
+                        for (int k = 0; k < sp.s; ++k)
+#pragma unroll
+                            for (int i = 0; i < CH; ++i) w[i] = mul2(w[i], add2(w[i], two2));
+#pragma unroll
+                        for (int i = 0; i < CH; ++i) w[i] = mul2(w[i], sW2);
+                    }
+#pragma unroll
+                    for (int i = 0; i < CH; ++i) {
+                        float a, b;
+                        upk2(w[i], a, b);
+                        split2<BF16>(a, b, H[h * CH + i], M[h * CH + i]);
+                    }
+                }
+            }
+            if (16 * (u + 1) == Kr) split2<BF16>(s21, -sW, H[7], M[7]);
+            tmem_st8(t_hi + u * 8, H);
+            tmem_st8(t_mid + u * 8, M);
+        }
+        tmem_st_wait();
+        tc_fence_before();
+        __syncwarp();
+        mbar_arrive_warp(&S->full[slot]);
+        ++stage;
         }
     }
     return true;
+}
+
+// One item, K and chunk count at run time.
+template <int KP, bool BF16, bool ALPHA>
+__device__ __forceinline__ bool gen_item_any(const Params &prm, Barriers *S, uint32_t &stage, uint32_t slot0, const ReqDesc &r,
+                                             const Item &it, uint32_t w_lane, int m) {
+    const SeriesPlan sp{uni(r.scaleW[1]), uni(r.scaleW[2])};
+    return sp.D == 3 ? gen_item<KP, BF16, 0, 0, ALPHA, 3>(prm, S, stage, slot0, r, it, sp, w_lane, m)
+         : sp.D == 5 ? gen_item<KP, BF16, 0, 0, ALPHA, 5>(prm, S, stage, slot0, r, it, sp, w_lane, m)
+                     : gen_item<KP, BF16, 0, 0, ALPHA, 8>(prm, S, stage, slot0, r, it, sp, w_lane, m);
+}
+
+// One item by the code for its K and chunk count: NEV chunks of regions and
+// the trough pair make K = 8 (NEV + 1) for an odd NEV, and 8 NEV or 8 (NEV + 2)
+// for an even one.
+template <int KP, bool BF16, int NEV>
+__device__ __forceinline__ bool gen_item_nev(const Params &prm, Barriers *S, uint32_t &stage, uint32_t slot0,
+                                             const ReqDesc &r, const Item &it, SeriesPlan sp, uint32_t w_lane, int m) {
+    constexpr int K0 = NEV % 2 ? 8 * (NEV + 1) : 8 * NEV, K1 = NEV % 2 == 0 && 8 * (NEV + 2) <= KP ? 8 * (NEV + 2) : K0;
+    if (K1 != K0 && uni(r.Kp == K1))
+        return sp.D == 3 ? gen_item<KP, BF16, K1, NEV, false, 3>(prm, S, stage, slot0, r, it, sp, w_lane, m)
+             : sp.D == 5 ? gen_item<KP, BF16, K1, NEV, false, 5>(prm, S, stage, slot0, r, it, sp, w_lane, m)
+                         : gen_item<KP, BF16, K1, NEV, false, 8>(prm, S, stage, slot0, r, it, sp, w_lane, m);
+    return sp.D == 3 ? gen_item<KP, BF16, K0, NEV, false, 3>(prm, S, stage, slot0, r, it, sp, w_lane, m)
+         : sp.D == 5 ? gen_item<KP, BF16, K0, NEV, false, 5>(prm, S, stage, slot0, r, it, sp, w_lane, m)
+                     : gen_item<KP, BF16, K0, NEV, false, 8>(prm, S, stage, slot0, r, it, sp, w_lane, m);
+}
+// Arguments above 0.55 (squarings) take the run-time form.
+template <int KP, bool BF16, bool FIXED>
+__device__ __forceinline__ bool gen_item_k(const Params &prm, Barriers *S, uint32_t &stage, uint32_t slot0,
+                                           const ReqDesc &r, const Item &it, uint32_t w_lane, int m) {
+    if constexpr (FIXED) {
+        constexpr int MAX_NEV = KP / 8;
+        const SeriesPlan sp{uni(r.scaleW[1]), uni(r.scaleW[2])};
+        if (sp.s == 0) {
+#define FG21_NEV(n) \
+    case n:         \
+        if constexpr (n <= MAX_NEV) return gen_item_nev<KP, BF16, n>(prm, S, stage, slot0, r, it, sp, w_lane, m);
+            switch (uni((r.N + 7) / 8)) {
+                FG21_NEV(1)
+                FG21_NEV(2)
+                FG21_NEV(3)
+                FG21_NEV(4)
+                FG21_NEV(5)
+                FG21_NEV(6)
+                FG21_NEV(7)
+                FG21_NEV(8)
+            }
+#undef FG21_NEV
+        }
+    }
+    return gen_item_any<KP, BF16, false>(prm, S, stage, slot0, r, it, w_lane, m);
 }
 
 // ------------------------------------------------------------- epilogue
-// tcgen05.ld of up to NB 16-column blocks of this thread's accumulator row.
-template <int NB>
-__device__ __forceinline__ void acc_issue(uint32_t taddr, int b0, int nb, float (&v)[NB][16]) {
-    tmem_ld16(taddr + b0 * 16, v[0]);
+// Sum of squares of 16-column accumulator blocks with packed FP32x2 FMAs:
+// accumulator pair k sums columns 2k, 2k+8 (low half) and 2k+1, 2k+9 (high half)
+// of every block, i.e. eight independent scalar chains in a fixed order,
+// combined by a fixed tree after every EPI_NB blocks (half the instructions of
+// scalar FMAs).
+template <bool FIRST>
+__device__ __forceinline__ void sq_block(uint64_t (&q)[4], const uint32_t *v) {
 #pragma unroll
-    for (int i = 1; i < NB; ++i)
-        if (nb > i) tmem_ld16(taddr + (b0 + i) * 16, v[i]);
-}
-// Sum of squares of NB 16-column blocks with packed FP32x2 FMAs: accumulator
-// pair k sums columns 2k, 2k+8 (low half) and 2k+1, 2k+9 (high half) of every
-// block, i.e. eight independent scalar chains in a fixed order, combined by a
-// fixed tree (half the instructions of scalar FMAs).
-template <int NB>
-__device__ __forceinline__ float acc_sumsq(const float (&v)[NB][16], int nb) {
-    uint64_t q[4] = {0, 0, 0, 0};
-#pragma unroll
-    for (int bb = 0; bb < NB; ++bb) {
-        if (bb < nb) {
-#pragma unroll
-            for (int jj = 0; jj < 16; jj += 2) {
-                const uint64_t x = pk2(v[bb][jj], v[bb][jj + 1]);
-                q[(jj >> 1) & 3] = fma2(x, x, q[(jj >> 1) & 3]);
-            }
-        }
+    for (int jj = 0; jj < 16; jj += 2) {
+        const uint64_t x = pk2(__uint_as_float(v[jj]), __uint_as_float(v[jj + 1]));
+        // the chains start with the bare square: x * x + 0
+        q[(jj >> 1) & 3] = FIRST && jj < 8 ? mul2(x, x) : fma2(x, x, q[(jj >> 1) & 3]);
     }
+}
+__device__ __forceinline__ float sq_tree(uint64_t (&q)[4]) {
     float a[8];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) upk2(q[k], a[2 * k], a[2 * k + 1]);
+    for (int k = 0; k < 4; ++k) {
+        upk2(q[k], a[2 * k], a[2 * k + 1]);
+    }
     return ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
 }
-
-// The epilogue of every stage of one item by one epilogue warp: per stage wait
-// for the MMAs (the accumulator), read and reduce this warp's half of the
-// t-blocks, release the accumulator slot; per item one compensated partial.
-template <bool RESID>
-__device__ __forceinline__ bool epi_item(const Params &prm, Barriers *S, Ring &rg, const ReqDesc &r, const Item &it,
-                                         uint32_t lane_addr, int half, int m) {
-    const int lane = threadIdx.x & 31;
-    const int64_t p = (int64_t)it.tile * 128 + m;
-    const bool in = p < r.P;
-    const int sWexp = *r.scaleW;
-    const int nch = r.n_tchunks, Tc = r.Tc, T = r.T, F = r.F;
-    const int nblk = r.Tc_pad / 16, hb = (nblk + 1) / 2;
-    const int b_lo = half * hb, b_hi = min(nblk, b_lo + hb);
-    const int *__restrict__ scaleB = r.scaleB;
-    float qs = 0.0f, qc = 0.0f;
-    int sb_n = __ldg(scaleB + it.f0 * nch);
-    for (int f = it.f0; f < it.f1; ++f) {
-        float qf = 0.0f;
-        for (int c = 0; c < nch; ++c) {
-            const int sb = sb_n;
-            sb_n = __ldg(scaleB + min(f * nch + c + 1, it.f1 * nch - 1));   // next stage's scale, one ahead
-            if (!mbar_wait(&S->done[rg.slot], rg.ph, S, prm.status, STATUS_TIMEOUT_EPI)) return false;
-            tc_fence_after();
-            const float unscale = exp2i(-(sWexp + sb));
-            const uint32_t taddr = lane_addr + rg.slot * prm.acc_cols;
-            float q = 0.0f;
-            for (int b0 = b_lo; b0 < b_hi; b0 += EPI_NB) {
-                const int nb = min(EPI_NB, b_hi - b0);
-                float v[EPI_NB][16];
-                acc_issue<EPI_NB>(taddr, b0, nb, v);
-                tmem_ld_wait();
-                if (RESID) {
-                    if (in) {
-                        const int t0 = c * Tc, tn = min(Tc, T - t0);
-                        for (int bb = 0; bb < nb; ++bb)
+// Loads NB (1 .. EPI_NB) blocks of this thread's accumulator row.
+template <int NB>
+__device__ __forceinline__ void acc_load(uint32_t taddr, uint32_t *v) {
+    if (NB >= 2) tmem_ld32(taddr, v);
+    else tmem_ld16(taddr, v);
+    if (NB == 3) tmem_ld16(taddr + 32, v + 32);
+    if (NB == 4) tmem_ld32(taddr + 32, v + 32);
+}
+template <int NB>
+__device__ __forceinline__ float acc_sumsq(const uint32_t *v) {
+    uint64_t q[4];
+    sq_block<true>(q, v);
 #pragma unroll
-                            for (int jj = 0; jj < 16; ++jj) {
-                                const int t = (b0 + bb) * 16 + jj;
-                                if (t < tn) prm.resid[((size_t)p * F + f) * T + t0 + t] = -v[bb][jj] * unscale;
-                            }
-                    }
-                } else {
-                    q += acc_sumsq<EPI_NB>(v, nb);
-                }
-            }
-            tc_fence_before();
-            __syncwarp();
-            mbar_arrive_warp(&S->full[rg.slot]);                 // accumulator free for stage + ring
-            rg.next(prm.ring);
-            qf += q * unscale * unscale;
+    for (int b = 1; b < NB; ++b) sq_block<false>(q, v + 16 * b);
+    return sq_tree(q);
+}
+// Sum of squares of NB blocks of this thread's accumulator row, a set of chains
+// for every EPI_NB of them; release() runs once they are in registers.
+template <int NB, typename Release>
+__device__ __forceinline__ float half_sumsq(uint32_t taddr, Release release) {
+    constexpr int N0 = NB < EPI_NB ? NB : EPI_NB, N1 = NB - N0;
+    float q = 0.0f;
+    if constexpr (NB > 0) {
+        uint32_t v[16 * EPI_NB];
+        acc_load<N0>(taddr, v);
+        tmem_ld_wait();
+        if constexpr (N1 > 0) {
+            q = acc_sumsq<N0>(v);
+            acc_load<N1>(taddr + 16 * EPI_NB, v);
+            tmem_ld_wait();
+            release();
+            q += acc_sumsq<N1>(v);
+        } else {
+            release();
+            q = acc_sumsq<N0>(v);
         }
-        kahan_add_dev(qs, qc, qf);
+    } else {
+        release();
     }
-    if (!RESID && in) r.partials[(size_t)p * r.n_part + 2 * it.g + half] = make_float2(qs, -qc);
-    return true;
+    return q;
 }
 
-// The MMA issuer's walk over its stages (items, channels, t-chunks) with the
-// per-item operand geometry.
-struct MmaStage {
-    int64_t item;
-    int f, c, f1, nch, ksteps, Kr, tc_pad;
-    uint32_t b_lbo, b_split;
-    Ring rg;
-    bool valid;
-    __device__ __forceinline__ void load_item(const Params &prm) {
-        valid = item < prm.n_items;
-        if (!valid) return;
-        const Item it = decode_item(prm.reqs, prm.n_reqs, item);
-        const ReqDesc &r = prm.reqs[it.req];
-        f = it.f0;
-        f1 = it.f1;
-        c = 0;
-        nch = r.n_tchunks;
-        Kr = r.Kp;
-        ksteps = Kr / 16;
-        b_lbo = (uint32_t)r.Tc_pad * 16;
-        b_split = (uint32_t)(Kr / 8) * b_lbo;
-        tc_pad = r.Tc_pad;
+// The epilogue of one item's stages by one warp (32 points): per stage wait for
+// the MMAs, read the accumulator row, release its slot, square and sum; per
+// item one compensated partial for each half of the t-blocks.
+template <bool RESID, int NBLK>
+__device__ __forceinline__ bool epi_item(const Params &prm, Barriers *S, uint32_t &stage, int lane_id,
+                                         const ReqDesc &r, const Item &it, uint32_t acc_lane, int m) {
+    const int64_t p = (int64_t)it.tile * 128 + m;
+    const int sWexp = *r.scaleW;
+    const int nch = uni(r.n_tchunks);
+    const int *__restrict__ scaleB = r.scaleB + it.f0 * nch;
+    const int n = (it.f1 - it.f0) * nch;
+    float qs0 = 0.0f, qc0 = 0.0f, qs1 = 0.0f, qc1 = 0.0f, qf0 = 0.0f, qf1 = 0.0f;
+    int sb_n = __ldg(scaleB), c = 0;
+    for (int k = 0; k < n; ++k) {
+        // 2^-(sW + sB), exponents within +-40 each
+        const float unscale = __int_as_float((127 - sWexp - sb_n) << 23);
+        sb_n = __ldg(scaleB + min(k + 1, n - 1));          // next stage's scale, one ahead
+        // the halves of the accumulator are written, read and freed one after the
+        // other, so that the next stage's first half can start while this one's
+        // second half is still read
+        constexpr int HB = (NBLK + 1) / 2;
+        float q0 = 0.0f, q1 = 0.0f;
+        if (!mbar_wait(&S->acc_done[lane_id], stage & 1u, S, prm.status, STATUS_TIMEOUT_EPI)) return false;
+        tc_fence_after();
+        auto release = [&](int h) {
+            tc_fence_before();
+            __syncwarp();
+            mbar_arrive_warp(&S->acc_free[2 * lane_id + h]);
+        };
+        if constexpr (!RESID) q0 = half_sumsq<HB>(acc_lane, [&] { release(0); });
+        if (!mbar_wait(&S->done[(lane_id << prm.ring_log2) + slot_of(stage, prm.ring_log2)],
+                       phase_of(stage, prm.ring_log2), S, prm.status, STATUS_TIMEOUT_EPI))
+            return false;
+        tc_fence_after();
+        if constexpr (RESID) {
+            const int Tc = r.Tc, T = r.T, F = r.F, nblk = r.Tc_pad / 16;
+            const int f = it.f0 + k / nch, t0 = (k % nch) * Tc, tn = min(Tc, T - t0);
+            for (int b = 0; b < nblk; ++b) {
+                uint32_t v[16];
+                tmem_ld16(acc_lane + b * 16, v);
+                tmem_ld_wait();
+                if (p < r.P)
+#pragma unroll
+                    for (int jj = 0; jj < 16; ++jj) {
+                        const int t = b * 16 + jj;
+                        if (t < tn) prm.resid[((size_t)p * F + f) * T + t0 + t] = -__uint_as_float(v[jj]) * unscale;
+                    }
+            }
+            release(0);
+            release(1);
+        } else {
+            q1 = half_sumsq<NBLK - HB>(acc_lane + 16 * HB, [&] { release(1); });
+        }
+        ++stage;
+        qf0 += q0 * unscale * unscale;
+        qf1 += q1 * unscale * unscale;
+        if (++c == nch) {
+            c = 0;
+            kahan_add_dev(qs0, qc0, qf0);
+            kahan_add_dev(qs1, qc1, qf1);
+            qf0 = qf1 = 0.0f;
+        }
     }
-    __device__ __forceinline__ void init(const Params &prm) {
-        item = blockIdx.x;
-        rg = Ring();
-        load_item(prm);
+    if (!RESID && p < r.P)
+        *reinterpret_cast<float4 *>(r.partials + (size_t)p * r.n_part + 2 * it.g) = make_float4(qs0, -qc0, qs1, -qc1);
+    return true;
+}
+// ... by the code for its block count (1 .. 12).
+template <bool RESID>
+__device__ __forceinline__ bool epi_item_n(const Params &prm, Barriers *S, uint32_t &stage, int lane_id,
+                                           const ReqDesc &r, const Item &it, uint32_t acc_lane, int m) {
+    static_assert(TC_MAX / 16 == 12, "one case per block count");
+    if constexpr (!RESID) {
+#define FG21_NBLK(n) \
+    case n: return epi_item<false, n>(prm, S, stage, lane_id, r, it, acc_lane, m);
+        switch (uni(r.Tc_pad / 16)) {
+            FG21_NBLK(2)
+            FG21_NBLK(3)
+            FG21_NBLK(4)
+            FG21_NBLK(5)
+            FG21_NBLK(6)
+            FG21_NBLK(7)
+            FG21_NBLK(8)
+            FG21_NBLK(9)
+            FG21_NBLK(10)
+            FG21_NBLK(11)
+            FG21_NBLK(12)
+        }
+#undef FG21_NBLK
     }
-    __device__ __forceinline__ void next(const Params &prm, int ring) {
-        rg.next(ring);
-        if (++c < nch) return;
-        c = 0;
-        if (++f < f1) return;
-        item += gridDim.x;
-        load_item(prm);
-    }
-};
+    return epi_item<RESID, 1>(prm, S, stage, lane_id, r, it, acc_lane, m);
+}
 
 // The stage's MMAs as straight-line code for KS k steps: the issuing thread
 // shares its scheduler with ALU warps, and loop control between the MMAs
@@ -685,8 +813,7 @@ struct MmaStage {
 // reduction adds back its expected half-ulp (chi2_scale).
 template <int KS>
 __device__ __forceinline__ void issue_mmas(uint32_t d_tmem, uint32_t w_hi, uint32_t w_mid, uint32_t b_addr,
-                                           uint32_t b_lbo, uint32_t b_split, uint32_t idesc) {
-#pragma unroll
+                                           uint32_t b_lbo, uint32_t b_split, uint32_t idesc, uint32_t el) {
     // one descriptor for the stage's tile; each MMA adds its offset (16-byte
     // units) to the start-address field, which shared-memory addresses below
     // 256 KB never carry out of (the issuing thread is busy about half the
@@ -695,51 +822,70 @@ __device__ __forceinline__ void issue_mmas(uint32_t d_tmem, uint32_t w_hi, uint3
     const uint32_t step = (2 * b_lbo) >> 4, split = b_split >> 4;
 #pragma unroll
     for (int ks = 0; ks < KS; ++ks) {
-        mma_f16_ts(d_tmem, w_hi + ks * 8, d0 + split + ks * step, idesc, ks > 0 ? 1u : 0u);
-        mma_f16_ts(d_tmem, w_mid + ks * 8, d0 + ks * step, idesc, 1u);
+        mma_f16_ts(d_tmem, w_hi + ks * 8, d0 + split + ks * step, idesc, ks > 0 ? 1u : 0u, el);
+        mma_f16_ts(d_tmem, w_mid + ks * 8, d0 + ks * step, idesc, 1u, el);
     }
 #pragma unroll
     for (int ks = KS - 1; ks >= 0; --ks)
-        mma_f16_ts(d_tmem, w_hi + ks * 8, d0 + ks * step, idesc, 1u);
+        mma_f16_ts(d_tmem, w_hi + ks * 8, d0 + ks * step, idesc, 1u, el);
 }
 
-template <int KP, bool BF16>
-__device__ __forceinline__ void issue_stage(const MmaStage &st, uint32_t tmem, uint32_t w_col0, char *b_slots,
-                                            const Params &prm) {
-    const uint32_t idesc = instr_desc(128, st.tc_pad, BF16);
-    const uint32_t w_hi = tmem + w_col0 + st.rg.slot * KP, w_mid = w_hi + st.Kr / 2;
-    const uint32_t b_addr = smem_u32(b_slots + st.rg.slot * prm.b_stage_bytes);
-    const uint32_t d_tmem = tmem + st.rg.slot * prm.acc_cols;
-    if (KP == 16 || st.ksteps == 1) issue_mmas<1>(d_tmem, w_hi, w_mid, b_addr, st.b_lbo, st.b_split, idesc);
-    else if (KP == 32 || st.ksteps == 2) issue_mmas<2>(d_tmem, w_hi, w_mid, b_addr, st.b_lbo, st.b_split, idesc);
-    else if (st.ksteps == 3) issue_mmas<3>(d_tmem, w_hi, w_mid, b_addr, st.b_lbo, st.b_split, idesc);
-    else issue_mmas<4>(d_tmem, w_hi, w_mid, b_addr, st.b_lbo, st.b_split, idesc);
+// The MMAs and commits of every stage of one item (KS k steps).  The columns of
+// a stage go in two halves (the epilogue's), each when its part of the
+// accumulator has been read.
+template <int KP, int KS, bool BF16>
+__device__ __forceinline__ bool mma_item(const Params &prm, Barriers *S, uint32_t &stage, int lane_id, int n, int tc_pad,
+                                         uint32_t tmem, uint32_t w_col0, uint32_t b_slots, uint32_t el) {
+    const int n0 = (tc_pad / 16 + 1) / 2 * 16, n1 = tc_pad - n0;       // columns of the halves (n1 may be 0)
+    const uint32_t idesc0 = instr_desc(128, n0, BF16), idesc1 = instr_desc(128, n1, BF16);
+    const uint32_t b_lbo = (uint32_t)tc_pad * 16, b_split = 2 * KS * b_lbo;
+    const uint32_t d = tmem + (uint32_t)(lane_id * prm.acc_cols);
+    for (int k = 0; k < n; ++k) {
+        const uint32_t slot = ((uint32_t)lane_id << prm.ring_log2) + slot_of(stage, prm.ring_log2);
+        const uint32_t w_hi = tmem + w_col0 + slot * KP, b = b_slots + slot * prm.b_stage_bytes;
+        if (!mbar_wait(&S->full[slot], phase_of(stage, prm.ring_log2), S, prm.status, STATUS_TIMEOUT_MMA) ||
+            !mbar_wait(&S->acc_free[2 * lane_id], (stage & 1u) ^ 1u, S, prm.status, STATUS_TIMEOUT_MMA))
+            return false;
+        tc_fence_after();
+        issue_mmas<KS>(d, w_hi, w_hi + 8 * KS, b, b_lbo, b_split, idesc0, el);
+        mma_commit(&S->acc_done[lane_id], el);
+        if (!mbar_wait(&S->acc_free[2 * lane_id + 1], (stage & 1u) ^ 1u, S, prm.status, STATUS_TIMEOUT_MMA))
+            return false;
+        tc_fence_after();
+        if (n1) issue_mmas<KS>(d + n0, w_hi, w_hi + 8 * KS, b + n0 * 16, b_lbo, b_split, idesc1, el);
+        mma_commit(&S->done[slot], el);
+        ++stage;
+    }
+    return true;
 }
 
-// Tensor-memory columns: accumulator of slot s at s * acc_cols; weights of
-// slot s at ring * acc_cols + s * KP (hi: Kr/2 columns, then mid: Kr/2).
+// Tensor-memory columns: accumulator of lane l at l * acc_cols; weights of slot
+// s after the accumulators, at s * KP (hi: Kr/2 columns, then mid: Kr/2).
 // RESID: validation mode (residuals of request 0 to prm.resid instead of the
 // chi2 partials); a separate instantiation keeps that code out of the
-// production kernel.  LEAN: every request of the launch has spectral-index
-// regions only (1: and K = KP, 2: K of any size), so the generators carry the
-// variants of their loop those requests need instead of all of them, each with
-// the series degree fixed per work item (smaller code: 5-9% faster).
-template <int KP, bool BF16, bool RESID, int LEAN>
+// production kernel.  ALPHA: some request of the launch has amplitude regions.
+template <int KP, bool BF16, bool RESID, bool ALPHA>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
     tc_loglike_kernel(const __grid_constant__ CUtensorMap tmap, const Params prm) {
     extern __shared__ __align__(1024) char smem_raw[];
     char *smem = reinterpret_cast<char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    const int ring = prm.ring;
+    const int ring = LANES << prm.ring_log2;
     char *b_slots = smem;                                             // [ring] x b_stage_bytes
     Barriers *S = reinterpret_cast<Barriers *>(b_slots + ring * prm.b_stage_bytes);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // broadcast, so that the compiler knows the role branches to be warp-uniform
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int s = 0; s < ring; ++s) {
             mbar_init(&S->full[s], FULL_ARRIVALS);
             mbar_init(&S->done[s], 1);
         }
-        mbar_init(&S->drain, 1);
+        for (int l = 0; l < LANES; ++l) {
+            mbar_init(&S->acc_done[l], 1);
+            mbar_init(&S->acc_free[2 * l], 4);       // the lane's epilogue warps
+            mbar_init(&S->acc_free[2 * l + 1], 4);
+            mbar_init(&S->drain[l], 1);
+        }
         S->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -755,115 +901,95 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     // the set-up above touches only this CTA's shared and tensor memory; from
     // here on the kernel reads what the operand pass wrote
     pdl_wait();
-    const uint32_t tmem = S->tmem_base;
-    const uint32_t w_col0 = (uint32_t)(ring * prm.acc_cols);
+    const uint32_t tmem = __shfl_sync(0xffffffffu, S->tmem_base, 0);
+    const uint32_t w_col0 = (uint32_t)(LANES * prm.acc_cols);
     const ReqDesc *__restrict__ reqs = prm.reqs;
 
-    if (warp < 8) {
+    if (warp < WARP_EPI) {
         // ================================================ weight generators
-        const int quad = warp & 3, half = warp >> 2;
-        const int m = quad * 32 + lane;
+        const int quad = warp & 3, lane_id = warp >> 2, m = quad * 32 + lane;
         const uint32_t w_lane = tmem + ((uint32_t)(quad * 32) << 16) + w_col0;
-        Ring rg;
+        const uint32_t slot0 = (uint32_t)lane_id << prm.ring_log2;
+        uint32_t stage = 0;
         bool ok = true;
-        GenItem<KP / 4> gi;
-        for (int64_t item = blockIdx.x; item < prm.n_items && ok; item += gridDim.x) {
+        for (int64_t item = first_item(lane_id); item < prm.n_items && ok; item += item_step()) {
             const Item it = decode_item(reqs, prm.n_reqs, item);
             const ReqDesc &r = reqs[it.req];
-            gen_item_load(gi, r, it, half, m);
-            // a request's Kr fixes the column count of each half; it must match its operand tiles
-            if (LEAN == 1 || (LEAN == 2 && gi.Kr == KP))
-                ok = gi.sp.D == 3 ? gen_item<KP, BF16, true, false, 3>(prm, S, rg, r, it, gi, w_lane, half)
-                   : gi.sp.D == 5 ? gen_item<KP, BF16, true, false, 5>(prm, S, rg, r, it, gi, w_lane, half)
-                                  : gen_item<KP, BF16, true, false, 8>(prm, S, rg, r, it, gi, w_lane, half);
-            else if (LEAN == 2)
-                ok = gi.sp.D == 3 ? gen_item<KP, BF16, false, false, 3>(prm, S, rg, r, it, gi, w_lane, half)
-                   : gi.sp.D == 5 ? gen_item<KP, BF16, false, false, 5>(prm, S, rg, r, it, gi, w_lane, half)
-                                  : gen_item<KP, BF16, false, false, 8>(prm, S, rg, r, it, gi, w_lane, half);
-            else if (r.Na) ok = gi.Kr == KP ? gen_item<KP, BF16, true, true>(prm, S, rg, r, it, gi, w_lane, half)
-                                            : gen_item<KP, BF16, false, true>(prm, S, rg, r, it, gi, w_lane, half);
-            else if (gi.Kr == KP) ok = gen_item<KP, BF16, true, false>(prm, S, rg, r, it, gi, w_lane, half);
-            else ok = gen_item<KP, BF16, false, false>(prm, S, rg, r, it, gi, w_lane, half);
+            if (ALPHA && r.Na) ok = gen_item_any<KP, BF16, true>(prm, S, stage, slot0, r, it, w_lane, m);
+            else ok = gen_item_k<KP, BF16, !BF16 && !RESID && !ALPHA>(prm, S, stage, slot0, r, it, w_lane, m);
         }
-    } else if (warp < 16) {
+    } else if (warp < WARP_TMA) {
         // ========================================================= epilogue
-        const int quad = warp & 3, half = (warp - 8) >> 2;
-        const int m = quad * 32 + lane;
-        const uint32_t lane_addr = tmem + ((uint32_t)(quad * 32) << 16);
-        // the accumulators of every slot start free: count their first release
-        if (lane == 0)
-            for (int sl = 0; sl < ring; ++sl) mbar_arrive(&S->full[sl]);
-        Ring rg;
+        const int quad = warp & 3, lane_id = (warp - WARP_EPI) >> 2, m = quad * 32 + lane;
+        const uint32_t acc_lane = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(lane_id * prm.acc_cols);
+        uint32_t stage = 0;
         bool ok = true;
-        for (int64_t item = blockIdx.x; item < prm.n_items && ok; item += gridDim.x) {
+        for (int64_t item = first_item(lane_id); item < prm.n_items && ok; item += item_step()) {
             const Item it = decode_item(reqs, prm.n_reqs, item);
-            ok = epi_item<RESID>(prm, S, rg, reqs[it.req], it, lane_addr, half, m);
+            ok = epi_item_n<RESID>(prm, S, stage, lane_id, reqs[it.req], it, acc_lane, m);
         }
-    } else if (warp == WARP_TMA) {
+    } else if (warp < WARP_MMA) {
         // ====================================================== TMA producer
+        // (the whole warp walks the lane's stages; its elected lane issues)
+        const int lane_id = warp - WARP_TMA;
+        const uint32_t el = elect_one(), slot0 = (uint32_t)lane_id << prm.ring_log2;
         bool ok = true;
-        Ring rg;
-        if (lane == 0) {
-            for (int64_t item = blockIdx.x; item < prm.n_items && ok; item += gridDim.x) {
-                const Item it = decode_item(reqs, prm.n_reqs, item);
-                const ReqDesc &r = reqs[it.req];
-                const int rows = (int)r.tile_rows, nch = r.n_tchunks;
-                const int64_t tile_row0 = r.tile_row0;
-                for (int f = it.f0; f < it.f1 && ok; ++f) {
-                    for (int c = 0; c < nch; ++c) {
-                        // the operand slot is free once the MMAs of stage - ring are done
-                        if (!mbar_wait(&S->done[rg.slot], rg.ph ^ 1, S, prm.status, STATUS_TIMEOUT_TMA)) { ok = false; break; }
-                        mbar_arrive_expect_tx(&S->full[rg.slot], (uint32_t)(rows * 128));
-                        const int64_t row0 = tile_row0 + (int64_t)(f * nch + c) * rows;
-                        char *dst = b_slots + rg.slot * prm.b_stage_bytes;
-                        for (int jr = 0; jr < rows; jr += prm.box_rows)
-                            tma_load_2d(dst + jr * 128, &tmap, 0, (int)(row0 + jr), &S->full[rg.slot]);
-                        rg.next(ring);
-                    }
+        uint32_t stage = 0;
+        for (int64_t item = first_item(lane_id); item < prm.n_items && ok; item += item_step()) {
+            const Item it = decode_item(reqs, prm.n_reqs, item);
+            const ReqDesc &r = reqs[it.req];
+            const int rows = uni((int)r.tile_rows), n = (it.f1 - it.f0) * uni(r.n_tchunks);
+            int row = uni((int)(r.tile_row0 + (int64_t)it.f0 * r.n_tchunks * r.tile_rows));
+            for (int k = 0; k < n; ++k) {
+                const uint32_t slot = slot0 + slot_of(stage, prm.ring_log2);
+                // the operand slot is free once the MMAs of stage - ring are done
+                if (!mbar_wait(&S->done[slot], phase_of(stage, prm.ring_log2) ^ 1u, S, prm.status,
+                               STATUS_TIMEOUT_TMA)) {
+                    ok = false;
+                    break;
                 }
+                mbar_arrive_expect_tx(&S->full[slot], (uint32_t)(rows * 128), el);
+                char *dst = b_slots + slot * prm.b_stage_bytes;
+                for (int jr = 0; jr < rows; jr += prm.box_rows)
+                    tma_load_2d(dst + jr * 128, &tmap, 0, row + jr, &S->full[slot], el);
+                row += rows;
+                ++stage;
             }
-            if (!ok) {
-                // copies already issued land within microseconds; give them time
-                // before the CTA (and its shared memory) goes away
-                const uint64_t t0 = globaltimer();
-                while (globaltimer() - t0 < 200000ull) {
-                }
+        }
+        if (!ok) {
+            // copies already issued land within microseconds; give them time
+            // before the CTA (and its shared memory) goes away
+            const uint64_t t0 = globaltimer();
+            while (globaltimer() - t0 < 200000ull) {
             }
         }
         __syncwarp();
     } else {
         // ========================================================= MMA issuer
-        // Stages are issued in pairs when the next one is already complete: a
-        // barrier operation right after a burst of MMAs stalls the issuing thread
-        // until they drain, so two stages' MMAs and commits go out back to back
-        // with the next stage's barrier tested (non-blocking) before the first.
+        // (the whole warp walks the lane's stages; its elected lane issues)
+        const int lane_id = warp - WARP_MMA;
+        const uint32_t el = elect_one(), b_addr = smem_u32(b_slots);
         bool ok = true;
-        if (lane == 0) {
-            MmaStage cur;
-            cur.init(prm);
-            while (cur.valid && ok) {
-                if (!mbar_wait(&S->full[cur.rg.slot], cur.rg.ph, S, prm.status, STATUS_TIMEOUT_MMA)) { ok = false; break; }
-                MmaStage nxt = cur;
-                nxt.next(prm, ring);
-                const bool pair = nxt.valid && mbar_test(&S->full[nxt.rg.slot], nxt.rg.ph);
-                tc_fence_after();
-                issue_stage<KP, BF16>(cur, tmem, w_col0, b_slots, prm);
-                mma_commit(&S->done[cur.rg.slot]);
-                if (pair) {
-                    issue_stage<KP, BF16>(nxt, tmem, w_col0, b_slots, prm);
-                    mma_commit(&S->done[nxt.rg.slot]);
-                    nxt.next(prm, ring);
-                }
-                cur = nxt;
-            }
-            // drain: every MMA issued so far completes before tensor memory is freed
-            mma_commit(&S->drain);
-            uint64_t t0 = globaltimer();
-            while (!mbar_try_wait(&S->drain, 0)) {
-                if (globaltimer() - t0 > WAIT_LIMIT_NS) {
-                    atomicOr(prm.status, STATUS_TIMEOUT_DRAIN);
-                    break;
-                }
+        uint32_t stage = 0;
+        for (int64_t item = first_item(lane_id); item < prm.n_items && ok; item += item_step()) {
+            const Item it = decode_item(reqs, prm.n_reqs, item);
+            const ReqDesc &r = reqs[it.req];
+            const int n = (it.f1 - it.f0) * uni(r.n_tchunks), tc_pad = uni(r.Tc_pad), ks = uni(r.Kp / 16);
+            if (KP == 16 || ks == 1)
+                ok = mma_item<KP, 1, BF16>(prm, S, stage, lane_id, n, tc_pad, tmem, w_col0, b_addr, el);
+            else if (KP == 32 || ks == 2)
+                ok = mma_item<KP, 2, BF16>(prm, S, stage, lane_id, n, tc_pad, tmem, w_col0, b_addr, el);
+            else if (ks == 3)
+                ok = mma_item<KP, 3, BF16>(prm, S, stage, lane_id, n, tc_pad, tmem, w_col0, b_addr, el);
+            else ok = mma_item<KP, 4, BF16>(prm, S, stage, lane_id, n, tc_pad, tmem, w_col0, b_addr, el);
+        }
+        // drain: every MMA issued so far completes before tensor memory is freed
+        mma_commit(&S->drain[lane_id], el);
+        const uint64_t t0 = globaltimer();
+        while (!mbar_try_wait(&S->drain[lane_id], 0)) {
+            if (globaltimer() - t0 > WAIT_LIMIT_NS) {
+                atomicOr(prm.status, STATUS_TIMEOUT_DRAIN);
+                break;
             }
         }
         __syncwarp();
@@ -889,33 +1015,32 @@ size_t smem_bytes(int ring, int b_stage_bytes) {
     return 1024 + (size_t)ring * b_stage_bytes + sizeof(Barriers) + 64;
 }
 
-template <int KP, bool BF16, bool RESID, int LEAN>
+template <int KP, bool BF16, bool RESID, bool ALPHA>
 cudaError_t launch_kpr(const CUtensorMap &map, const Params &prm, int grid, size_t sm, cudaStream_t stream) {
     static bool attr = false;
     if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(tc_loglike_kernel<KP, BF16, RESID, LEAN>,
+        cudaError_t e = cudaFuncSetAttribute(tc_loglike_kernel<KP, BF16, RESID, ALPHA>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
         if (e != cudaSuccess) return e;
         attr = true;
     }
-    cudaError_t e = launch_dependent(tc_loglike_kernel<KP, BF16, RESID, LEAN>, dim3(grid), dim3(NUM_THREADS), sm,
+    cudaError_t e = launch_dependent(tc_loglike_kernel<KP, BF16, RESID, ALPHA>, dim3(grid), dim3(NUM_THREADS), sm,
                                      stream, map, prm);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
 
 template <int KP, bool BF16>
-cudaError_t launch_kp(const CUtensorMap &map, const Params &prm, int grid, size_t sm, int lean,
+cudaError_t launch_kp(const CUtensorMap &map, const Params &prm, int grid, size_t sm, bool alpha,
                       cudaStream_t stream) {
-    if (prm.resid) return launch_kpr<KP, BF16, true, 0>(map, prm, grid, sm, stream);
-    if (lean == 1) return launch_kpr<KP, BF16, false, 1>(map, prm, grid, sm, stream);
-    if (lean == 2 && KP > 16) return launch_kpr<KP, BF16, false, 2>(map, prm, grid, sm, stream);
-    return launch_kpr<KP, BF16, false, 0>(map, prm, grid, sm, stream);
+    if (prm.resid) return launch_kpr<KP, BF16, true, true>(map, prm, grid, sm, stream);
+    if (alpha) return launch_kpr<KP, BF16, false, true>(map, prm, grid, sm, stream);
+    return launch_kpr<KP, BF16, false, false>(map, prm, grid, sm, stream);
 }
 
 cudaError_t launch_common(const ReqDesc *d_reqs, int n_reqs, int64_t n_items, int kp_max, int tc_pad_max,
                           int precision, void *arena, int64_t arena_rows, unsigned *status, float *resid,
-                          int box_rows, int num_sms, int lean, cudaStream_t stream) {
+                          int box_rows, int num_sms, bool alpha, cudaStream_t stream) {
     if (n_items == 0) return cudaSuccess;
     if (tc_map_init() != FG21_OK) return cudaErrorNotSupported;
     CUtensorMap map;
@@ -936,16 +1061,16 @@ cudaError_t launch_common(const ReqDesc *d_reqs, int n_reqs, int64_t n_items, in
     prm.n_items = n_items;
     prm.b_stage_bytes = ((4 * kp_max * tc_pad_max) + 1023) & ~1023;
     prm.acc_cols = tc_pad_max;
-    // as many stage slots (accumulator + weights in tensor memory) as fit, 2..4
-    const int per_slot = tc_pad_max + kp;
-    int ring = 512 / per_slot;
-    if (ring > MAX_RING) ring = MAX_RING;
-    if (ring < 2) return cudaErrorInvalidValue;
-    // ... and as fit shared memory next to the barriers
-    while (ring > 2 && smem_bytes(ring, prm.b_stage_bytes) > 227 * 1024) --ring;
-    prm.ring = ring;
+    // Tensor memory, for each of the two lanes: an accumulator (used in halves),
+    // and 4, 2 or 1 stage slots as the rest and shared memory (operand tiles,
+    // barriers) hold.
+    prm.ring_log2 = 2;
+    while (prm.ring_log2 > 0 && (LANES * tc_pad_max + ((LANES * kp) << prm.ring_log2) > 512 ||
+                                 smem_bytes(LANES << prm.ring_log2, prm.b_stage_bytes) > 227 * 1024))
+        --prm.ring_log2;
+    const int ring = LANES << prm.ring_log2;
     uint32_t cols = 32;
-    while (cols < (uint32_t)(ring * per_slot)) cols *= 2;
+    while (cols < (uint32_t)(LANES * tc_pad_max + ring * kp)) cols *= 2;
     if (cols > 512) return cudaErrorInvalidValue;
     prm.tmem_cols = cols;
     prm.status = status;
@@ -958,13 +1083,13 @@ cudaError_t launch_common(const ReqDesc *d_reqs, int n_reqs, int64_t n_items, in
     const int grid = (int)(n_items < num_sms ? n_items : num_sms);
     const bool bf16 = precision == FG21_PREC_BF16X3;
     if (kp == 16)
-        return bf16 ? launch_kp<16, true>(map, prm, grid, sm, lean, stream)
-                    : launch_kp<16, false>(map, prm, grid, sm, lean, stream);
+        return bf16 ? launch_kp<16, true>(map, prm, grid, sm, alpha, stream)
+                    : launch_kp<16, false>(map, prm, grid, sm, alpha, stream);
     if (kp == 32)
-        return bf16 ? launch_kp<32, true>(map, prm, grid, sm, lean, stream)
-                    : launch_kp<32, false>(map, prm, grid, sm, lean, stream);
-    return bf16 ? launch_kp<64, true>(map, prm, grid, sm, lean, stream)
-                : launch_kp<64, false>(map, prm, grid, sm, lean, stream);
+        return bf16 ? launch_kp<32, true>(map, prm, grid, sm, alpha, stream)
+                    : launch_kp<32, false>(map, prm, grid, sm, alpha, stream);
+    return bf16 ? launch_kp<64, true>(map, prm, grid, sm, alpha, stream)
+                : launch_kp<64, false>(map, prm, grid, sm, alpha, stream);
 }
 
 // Self-test of the bounded waits, on barriers that nothing ever arrives on.
@@ -1038,9 +1163,10 @@ __global__ void __launch_bounds__(128, 1) mma_probe_kernel(const uint16_t *__res
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (tid == 0) {
-        mma_f16_ts(tm, tm + 16, smem_desc(smem_u32(&sb[0][0][0]), 16 * 16, 128), instr_desc(128, 16, false), 1u);
-        mma_commit(&bar);
+    if (warp == 0) {
+        const uint32_t el = elect_one();
+        mma_f16_ts(tm, tm + 16, smem_desc(smem_u32(&sb[0][0][0]), 16 * 16, 128), instr_desc(128, 16, false), 1u, el);
+        mma_commit(&bar, el);
     }
     const uint64_t t0 = globaltimer();
     bool ok = true;
@@ -1052,11 +1178,11 @@ __global__ void __launch_bounds__(128, 1) mma_probe_kernel(const uint16_t *__res
         }
     }
     tc_fence_after();
-    float r[16];
+    uint32_t r[16];
     tmem_ld16(lane_base, r);
     tmem_ld_wait();
 #pragma unroll
-    for (int n = 0; n < 16; ++n) d[tid * 16 + n] = ok ? r[n] : __int_as_float(0x7FC00000);
+    for (int n = 0; n < 16; ++n) d[tid * 16 + n] = ok ? __uint_as_float(r[n]) : __int_as_float(0x7FC00000);
     tc_fence_before();
     __syncthreads();
     if (warp == 0) {
@@ -1115,7 +1241,7 @@ int tc_box_rows(const int64_t *tile_rows, int n) {
 
 cudaError_t launch_tc(const TcLaunch &L, int num_sms, cudaStream_t stream) {
     return launch_common(L.d_reqs, L.n_reqs, L.n_items, L.kp_max, L.tc_pad_max, L.precision, L.arena,
-                         L.arena_rows, L.status, nullptr, L.box_rows, num_sms, L.lean, stream);
+                         L.arena_rows, L.status, nullptr, L.box_rows, num_sms, L.alpha, stream);
 }
 
 cudaError_t launch_tc_residuals(const ReqDesc *h_req, const ReqDesc *d_req, int precision, float *resid,
@@ -1130,7 +1256,7 @@ cudaError_t launch_tc_residuals(const ReqDesc *h_req, const ReqDesc *d_req, int 
     const int64_t rows = h_req->tile_row0 + (int64_t)h_req->F * h_req->n_tchunks * h_req->tile_rows;
     const int64_t items = (int64_t)h_req->n_tiles * h_req->G;
     return launch_common(d_req, 1, items, h_req->Kp, h_req->Tc_pad, precision, arena, rows, h_req->status, resid,
-                         tc_box_rows(&h_req->tile_rows, 1), sms, 0, stream);
+                         tc_box_rows(&h_req->tile_rows, 1), sms, true, stream);
 }
 
 }  // namespace fg21
