@@ -79,7 +79,7 @@ int fg21_graph_create_multi(fg21_model *const *models, const double *const *d_pa
         return rc;
     }
     // descriptors once, outside the graph
-    cudaError_t e = cudaMemcpy(g->ws.d_reqs, g->ws.pinned, sizeof(ReqDesc) * g->reqs.size(), cudaMemcpyHostToDevice);
+    cudaError_t e = cudaMemcpy(g->ws.d_reqs, g->reqs.data(), sizeof(ReqDesc) * g->reqs.size(), cudaMemcpyHostToDevice);
     cudaStream_t s = nullptr;
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);

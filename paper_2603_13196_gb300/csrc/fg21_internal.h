@@ -145,8 +145,10 @@ ReqLayout request_layout(const ReqDesc &r, int precision);
 
 // ------------------------------------------------------- kernel launchers
 // All enqueue on `stream` and return cudaError_t of the launch.
-cudaError_t launch_prep(const ReqDesc *h_reqs, const ReqDesc *d_reqs, int n_reqs, int precision,
-                        int max_stat_blocks, int max_F_chunks, int max_tiles, cudaStream_t stream);
+// launch_prep also clears the status block, and stores a single request's
+// descriptor at d_reqs (`store`); several requests' descriptors must be there.
+cudaError_t launch_prep(const ReqDesc *h_reqs, ReqDesc *d_reqs, int n_reqs, int precision, int max_stat_blocks,
+                        int max_F_chunks, int max_tiles, bool store, cudaStream_t stream);
 cudaError_t launch_simt(const ReqDesc *h_reqs, const ReqDesc *d_reqs, int n_reqs, int precision,
                         cudaStream_t stream);
 // Blocks of the SIMT kernel of `precision` that one SM holds at once for a

@@ -36,6 +36,16 @@ constexpr int FIN_GROUP_SCRATCH = 512;   // floats of per-group finalise results
 __host__ __device__ inline int prep_head_doubles(int NP) {
     return NP + (2 * NP + 2 + 16 + 1) / 2 + FIN_GROUP_SCRATCH / 2;
 }
+// Requests without a statistics pass of their own on the tensor path (see prep_tc_kernel).
+constexpr int FUSED_POINTS = 256, FUSED_VALUES = 4096;
+__host__ __device__ inline bool request_fused(const ReqDesc &r) {
+    return r.coef2 && r.P <= FUSED_POINTS && r.P * (r.NPF + 4) <= FUSED_VALUES;
+}
+// Start of a block's slab after the staged rows and validity bytes (16-byte aligned).
+__host__ __device__ inline size_t fused_doubles(int P, int Rp) {
+    return ((size_t)P * Rp + (P + 7) / 8 + 1) / 2 * 2;
+}
+__device__ __forceinline__ double *fused_slab(double *base, int P, int Rp) { return base + fused_doubles(P, Rp); }
 constexpr int REDUCE_THREADS = 64;
 constexpr int REDUCE_SERIAL_MAX = 32;       // longest partial row summed by one thread
 
@@ -204,10 +214,9 @@ struct Fin {
     float nv, ma, x;
     int sW;
 };
-__device__ Fin prep_finalize(const ReqDesc &r, float *sh /* [2 NPF + 2 + 2 nwarps] */,
-                             float *gpart /* [FIN_GROUP_SCRATCH] */, double *bbar_sh, bool publish) {
-    const int N = r.NPF, Nb = r.Nb, nb = r.n_stat_blocks, W = 2 * N + 2;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+__device__ __forceinline__ void gather_stats(const ReqDesc &r, float *sh /* [2 NPF + 2] */,
+                                             float *gpart /* [FIN_GROUP_SCRATCH] */) {
+    const int N = r.NPF, nb = r.n_stat_blocks, W = 2 * N + 2;
     const int G = max(1, min((int)blockDim.x / W, FIN_GROUP_SCRATCH / W));
     for (int idx = threadIdx.x; idx < G * W; idx += blockDim.x) {
         const int g = idx / W, j = idx - g * W;
@@ -234,6 +243,41 @@ __device__ Fin prep_finalize(const ReqDesc &r, float *sh /* [2 NPF + 2 + 2 nwarp
         }
         sh[j] = v;
     }
+}
+// The same fields of a request of at most FUSED_POINTS points from its parameter
+// rows in shared memory ([P][Rp]; one thread per point tests it, then one warp
+// per field), by the same conversions and minima as the statistics blocks.
+// `valid` [FUSED_POINTS] bytes.
+__device__ __forceinline__ void row_stats(const ReqDesc &r, const double *rows, int Rp, float *sh,
+                                          unsigned char *valid) {
+    const int N = r.NPF, P = (int)r.P, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    for (int p = threadIdx.x; p < P; p += blockDim.x) valid[p] = point_valid(rows + (size_t)p * Rp, r);
+    __syncthreads();
+    for (int i = warp; i <= N; i += nw) {        // fields 0 .. NPF-1, then the trough amplitude and the count
+        float mn = INFINITY, mx = -INFINITY;
+        int n = 0;
+        for (int p = lane; p < P; p += 32)
+            if (valid[p]) {
+                const float b = f32_of_f64(rows[(size_t)p * Rp + i]);
+                mn = fminf(mn, b);
+                mx = fmaxf(mx, i < N ? b : fabsf(b));
+                ++n;
+            }
+        mn = warp_min(mn);
+        mx = warp_max(mx);
+        n = __reduce_add_sync(0xffffffffu, n);
+        if (lane == 0) {
+            // with no valid point the amplitude's maximum is 0, as the statistics blocks have it
+            sh[2 * i] = i < N ? mn : (float)n;
+            sh[2 * i + 1] = i < N || n > 0 ? mx : 0.0f;
+        }
+    }
+}
+// The rest of the finalise from the request's fields in `sh` ([2 NPF + 2 + 2
+// nwarps]): reference point, argument bound, scale and series.
+__device__ __forceinline__ Fin finish_stats(const ReqDesc &r, float *sh, double *bbar_sh, bool publish) {
+    const int N = r.NPF, Nb = r.Nb, W = 2 * N + 2;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     __syncthreads();
     const float nv = sh[2 * N], ma = sh[2 * N + 1];
     float dev = 0.0f, gdev = 0.0f;
@@ -280,13 +324,37 @@ __device__ Fin prep_finalize(const ReqDesc &r, float *sh /* [2 NPF + 2 + 2 nwarp
     __syncthreads();
     return f;
 }
+__device__ __forceinline__ Fin prep_finalize(const ReqDesc &r, float *sh, float *gpart, double *bbar_sh, bool publish) {
+    gather_stats(r, sh, gpart);
+    return finish_stats(r, sh, bbar_sh, publish);
+}
 
-__global__ void __launch_bounds__(STAT_BLOCK) prep_stats_kernel(const ReqDesc *__restrict__ reqs, int staged) {
+// Start of a call, by one block: the status word and the invalid counter are
+// cleared, and a single request's descriptor, which reaches this kernel as an
+// argument, is stored for the kernels after it (no copy, no memset and no host
+// staging buffer in the way of a call: 64 points, 3 regions: 27 us a call with
+// them).
+__device__ __forceinline__ void begin_call(const ReqDesc &r, ReqDesc *store) {
+    if (threadIdx.x < 8) r.status[threadIdx.x] = 0;
+    if (store) {
+        const uint64_t *src = reinterpret_cast<const uint64_t *>(&r);
+        for (int i = threadIdx.x; i < (int)(sizeof(ReqDesc) / 8); i += blockDim.x)
+            reinterpret_cast<uint64_t *>(store)[i] = src[i];
+    }
+}
+static_assert(sizeof(ReqDesc) % 8 == 0 && sizeof(ReqDesc) <= 2048, "the descriptor travels as a kernel argument");
+
+// ONE: the launch's only request, passed by value (stored at `store` unless
+// null); otherwise reqs[blockIdx.y].
+template <bool ONE>
+__global__ void __launch_bounds__(STAT_BLOCK) prep_stats_kernel(const ReqDesc *__restrict__ reqs, int staged,
+                                                                const __grid_constant__ ReqDesc one, ReqDesc *store) {
     // shared: [STAT_BLOCK / 32][2 NPF + 2] FP32 warp partials, then (staged) the
     // block's parameter rows [STAT_BLOCK][padded_row(NPF + 4)] FP64
     extern __shared__ double sh_stats_d[];     // [STAT_BLOCK / 32][2 NPF + 2] partials, then the rows
-    const ReqDesc &r = reqs[blockIdx.y];
-    if ((int)blockIdx.x >= r.n_stat_blocks) return;
+    const ReqDesc &r = ONE ? one : reqs[blockIdx.y];
+    if (blockIdx.x == 0 && blockIdx.y == 0) begin_call(r, ONE ? store : nullptr);
+    if ((int)blockIdx.x >= r.n_stat_blocks || request_fused(r)) return;
     const int N = r.NPF, W = 2 * N + 2, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nw = blockDim.x >> 5;
     float *sh_stats = reinterpret_cast<float *>(sh_stats_d);
@@ -366,8 +434,9 @@ __global__ void __launch_bounds__(STAT_BLOCK) prep_stats_kernel(const ReqDesc *_
 // Two threads per point (`half` 0 and 1 of the block): the deviation rows
 // alternate between them; half 0 also writes the trough rows and the sigma_n
 // terms, half 1 the amplitude rows.  `th` is the point's parameter row (staged
-// in shared memory).
-__device__ __forceinline__ void prep_points(const ReqDesc &r, int tile, const double *bbar, const double *th) {
+// in shared memory), `valid` its validity.
+__device__ __forceinline__ void prep_points(const ReqDesc &r, int tile, const double *bbar, const double *th,
+                                            bool valid) {
     const int pidx = threadIdx.x % TILE_M, half = threadIdx.x / TILE_M;
     if (half > 1) return;
     const int64_t p = (int64_t)tile * TILE_M + pidx;
@@ -394,7 +463,7 @@ __device__ __forceinline__ void prep_points(const ReqDesc &r, int tile, const do
         const float s21 = in ? f32_of_f64(th[NP + 2]) : 1.0f;
         out[(size_t)Kp * TILE_M] = 1.0f / (2.0f * s21 * s21);
         // the sigma_n terms of eq. likelihood for the reduction (FP64, once per point)
-        if (in && r.pvalid[p]) {
+        if (valid) {
             const double sig = th[NP + 3];
             r.pnorm[p] = make_double2((double)r.F * (double)r.T * log(2.0 * 3.141592653589793 * sig * sig),
                                       1.0 / (sig * sig));
@@ -519,17 +588,28 @@ __global__ void __launch_bounds__(PREP_THREADS) prep_tiles_kernel(const ReqDesc 
 // column of the weights), row Kp-1 holds dref 2^sB (multiplies -1), other rows
 // and columns t >= Tc are zero.
 //
-// Shared memory: bbar [NPF], finalise scratch and group results, then the block's slab --
+// A request of at most FUSED_POINTS points and FUSED_VALUES parameter values has
+// no statistics pass: every block stages all its rows and takes the statistics
+// itself (the same values), which costs each block less than the extra launch:
+// a call of 64 points and 3 regions takes 18.5 us against 22.7, 200 points and 12
+// regions 18.8 against 22.6, 256 points and 12 regions (4096 values, 32 KB of rows
+// a block) 20.6 against 22.6.  At 400 points and 14 regions (7200 values) the two
+// are equal, at 1000 points and 10 regions staging costs 19 us.
+//
+// Shared memory: bbar [NPF], finalise scratch and group results, then (fused
+// statistics) the request's rows and validity bytes, then the block's slab --
 // channel: the products' hi and lo parts [N][Tc_pad] each, E hi / lo and dref
 // [Tc_pad], wbar hi / lo [N] (FP32); points: parameter rows
 // [128][padded_row(NPF+4)] FP64.
-template <bool BF16>
-__global__ void __launch_bounds__(PREP_THREADS) prep_tc_kernel(const ReqDesc *__restrict__ reqs) {
+template <bool BF16, bool ONE>
+__global__ void __launch_bounds__(PREP_THREADS) prep_tc_kernel(const ReqDesc *__restrict__ reqs, int begin,
+                                                               const __grid_constant__ ReqDesc one, ReqDesc *store) {
     extern __shared__ double smem_d[];
     __shared__ float sh_red[PREP_THREADS / 32];
     __shared__ int s_scaleB;
     pdl_wait();
-    const ReqDesc &r = reqs[blockIdx.y];
+    const ReqDesc &r = ONE ? one : reqs[blockIdx.y];
+    if (begin && blockIdx.x == 0 && blockIdx.y == 0) begin_call(r, ONE ? store : nullptr);
     const int nfc = r.F * r.n_tchunks;
     if ((int)blockIdx.x >= nfc + r.n_tiles) return;
     const int N = r.N, NP = r.NPF, Nb = r.Nb, T = r.T;
@@ -537,19 +617,35 @@ __global__ void __launch_bounds__(PREP_THREADS) prep_tc_kernel(const ReqDesc *__
     float *fin_sh = reinterpret_cast<float *>(bbar + NP);
     float *gpart = reinterpret_cast<float *>(bbar + NP + (2 * NP + 2 + 16 + 1) / 2);
     double *slab = bbar + prep_head_doubles(NP);
+    const bool fused = request_fused(r);
+    const int R = NP + 4, Rp = padded_row(R);
+    double *rows = slab;                               // fused statistics: [P][Rp] rows, then [P] validity bytes
+    unsigned char *valid = reinterpret_cast<unsigned char *>(rows + (size_t)r.P * Rp);
+    if (fused) {
+        copy_rows8(rows, Rp, r.params, R, (int)r.P);
+        slab = fused_slab(slab, (int)r.P, Rp);
+    }
     if ((int)blockIdx.x >= nfc) {
         // ---- per-point operands of one 128-point tile
         const int tile = blockIdx.x - nfc;
         const int64_t p0 = (int64_t)tile * TILE_M;
         const int np = (int)min((int64_t)TILE_M, r.P - p0);
-        const int R = NP + 4, Rp = padded_row(R);
-        const double *src = r.params + p0 * R;
-        copy_rows8(slab, Rp, src, R, np);
-        prep_finalize(r, fin_sh, gpart, bbar, false);
-        cp_async_wait_all();
-        __syncthreads();
         const int pidx = threadIdx.x % TILE_M;
-        prep_points(r, tile, bbar, slab + (size_t)(pidx < np ? pidx : 0) * Rp);
+        if (fused) {
+            cp_async_wait_all();
+            __syncthreads();
+            row_stats(r, rows, Rp, fin_sh, valid);
+            finish_stats(r, fin_sh, bbar, false);
+            if ((int)threadIdx.x < np) r.pvalid[p0 + threadIdx.x] = valid[p0 + threadIdx.x];
+            prep_points(r, tile, bbar, rows + (size_t)(p0 + (pidx < np ? pidx : 0)) * Rp,
+                        pidx < np && valid[p0 + pidx]);
+        } else {
+            copy_rows8(slab, Rp, r.params + p0 * R, R, np);
+            prep_finalize(r, fin_sh, gpart, bbar, false);
+            cp_async_wait_all();
+            __syncthreads();
+            prep_points(r, tile, bbar, slab + (size_t)(pidx < np ? pidx : 0) * Rp, pidx < np && r.pvalid[p0 + pidx]);
+        }
         return;
     }
     // ---- operand tile of one (channel, t-chunk), in double-float arithmetic
@@ -577,7 +673,15 @@ __global__ void __launch_bounds__(PREP_THREADS) prep_tc_kernel(const ReqDesc *__
         cp_async4(eh + t, r.E_hi + ft0 + t);
         cp_async4(el + t, r.E_lo + ft0 + t);
     }
-    const Fin fin = prep_finalize(r, fin_sh, gpart, bbar, fc == 0);
+    Fin fin;
+    if (fused) {
+        cp_async_wait_all();
+        __syncthreads();
+        row_stats(r, rows, Rp, fin_sh, valid);
+        fin = finish_stats(r, fin_sh, bbar, fc == 0);
+    } else {
+        fin = prep_finalize(r, fin_sh, gpart, bbar, fc == 0);
+    }
     const double L = r.L[f];
     if (c == 0 && threadIdx.x == 32) {
         // the generators' series coefficients for this channel (the same FP32
@@ -1113,25 +1217,36 @@ cudaError_t opt_in_smem(K kernel, size_t need, size_t &current) {
     return e;
 }
 
-cudaError_t launch_prep(const ReqDesc *h_reqs, const ReqDesc *d_reqs, int n_reqs, int precision,
-                        int max_stat_blocks, int max_F_chunks, int max_tiles, cudaStream_t stream) {
+cudaError_t launch_prep(const ReqDesc *h_reqs, ReqDesc *d_reqs, int n_reqs, int precision, int max_stat_blocks,
+                        int max_F_chunks, int max_tiles, bool store, cudaStream_t stream) {
     int maxNP = 0;
-    for (int k = 0; k < n_reqs; ++k) maxNP = maxNP > h_reqs[k].NPF ? maxNP : h_reqs[k].NPF;
+    bool stats = false;                 // some request takes the statistics pass
+    for (int k = 0; k < n_reqs; ++k) {
+        maxNP = maxNP > h_reqs[k].NPF ? maxNP : h_reqs[k].NPF;
+        stats = stats || !request_fused(h_reqs[k]);
+    }
     // the finalise keeps one row of statistics per thread group in FIN_GROUP_SCRATCH
     // floats (2 NPF + 2 <= 256 within the documented region limits)
     if (2 * maxNP + 2 > FIN_GROUP_SCRATCH) return cudaErrorInvalidValue;
-    dim3 g1(max_stat_blocks, n_reqs);
-    // warp partials, then the staged parameter rows when they fit comfortably
-    const size_t part = sizeof(double) * (((size_t)(STAT_BLOCK / 32) * (2 * maxNP + 2) + 1) / 2);
-    const size_t slab1 = sizeof(double) * (size_t)STAT_BLOCK * padded_row(maxNP + 4);
-    const int staged = slab1 <= 96 * 1024;
-    const size_t sm1 = part + (staged ? slab1 : 0);
-    static size_t stats_opt_in = 48 * 1024;
-    cudaError_t e = opt_in_smem(prep_stats_kernel, sm1, stats_opt_in);
-    if (e != cudaSuccess) return e;
-    prep_stats_kernel<<<g1, STAT_BLOCK, sm1, stream>>>(d_reqs, staged);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    const bool one = n_reqs == 1;
+    ReqDesc *dst = store && one ? d_reqs : nullptr;
+    cudaError_t e = cudaSuccess;
+    if (stats) {
+        dim3 g1(max_stat_blocks, n_reqs);
+        // warp partials, then the staged parameter rows when they fit comfortably
+        const size_t part = sizeof(double) * (((size_t)(STAT_BLOCK / 32) * (2 * maxNP + 2) + 1) / 2);
+        const size_t slab1 = sizeof(double) * (size_t)STAT_BLOCK * padded_row(maxNP + 4);
+        const int staged = slab1 <= 96 * 1024;
+        const size_t sm1 = part + (staged ? slab1 : 0);
+        static size_t stats_opt_in[2] = {48 * 1024, 48 * 1024};
+        e = one ? opt_in_smem(prep_stats_kernel<true>, sm1, stats_opt_in[1])
+                : opt_in_smem(prep_stats_kernel<false>, sm1, stats_opt_in[0]);
+        if (e != cudaSuccess) return e;
+        if (one) prep_stats_kernel<true><<<g1, STAT_BLOCK, sm1, stream>>>(d_reqs, staged, h_reqs[0], dst);
+        else prep_stats_kernel<false><<<g1, STAT_BLOCK, sm1, stream>>>(d_reqs, staged, h_reqs[0], nullptr);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
     const bool tc = precision == FG21_PREC_FP16X3 || precision == FG21_PREC_BF16X3;
     size_t sm = 0;
     for (int k = 0; k < n_reqs; ++k) {
@@ -1140,25 +1255,30 @@ cudaError_t launch_prep(const ReqDesc *h_reqs, const ReqDesc *d_reqs, int n_reqs
         size_t need;
         if (tc) {
             const size_t chan = sizeof(float) * (2 * (size_t)r.N * r.Tc_pad + 3 * (size_t)r.Tc_pad + 2 * (size_t)r.N);
-            const size_t pts = sizeof(double) * (size_t)TILE_M * padded_row(r.NPF + 4);
-            need = head + (chan > pts ? chan : pts);
+            const int Rp = padded_row(r.NPF + 4);
+            const size_t pts = sizeof(double) * (size_t)TILE_M * Rp;
+            need = request_fused(r) ? head + sizeof(double) * fused_doubles((int)r.P, Rp) + chan
+                                    : head + (chan > pts ? chan : pts);
         } else {
             need = head + sizeof(double) * (size_t)r.N;
         }
         sm = sm > need ? sm : need;
     }
     dim3 g2(max_F_chunks + max_tiles, n_reqs);
-    static size_t tc_opt_in[2] = {48 * 1024, 48 * 1024};
-    if (precision == FG21_PREC_FP16X3) e = opt_in_smem(prep_tc_kernel<false>, sm, tc_opt_in[0]);
-    if (precision == FG21_PREC_BF16X3) e = opt_in_smem(prep_tc_kernel<true>, sm, tc_opt_in[1]);
-    if (e != cudaSuccess) return e;
-    switch (precision) {
-        case FG21_PREC_FP16X3: e = launch_dependent(prep_tc_kernel<false>, g2, PREP_THREADS, sm, stream, d_reqs); break;
-        case FG21_PREC_BF16X3: e = launch_dependent(prep_tc_kernel<true>, g2, PREP_THREADS, sm, stream, d_reqs); break;
-        case FG21_PREC_FP32_DELTA:
-            e = launch_dependent(prep_tiles_kernel<2>, g2, PREP_THREADS, sm, stream, d_reqs);
-            break;
-        default: e = launch_dependent(prep_tiles_kernel<3>, g2, PREP_THREADS, sm, stream, d_reqs); break;
+    if (tc) {
+        const bool bf = precision == FG21_PREC_BF16X3;
+        static size_t tc_opt_in[4] = {48 * 1024, 48 * 1024, 48 * 1024, 48 * 1024};
+        auto *kernel = bf ? (one ? prep_tc_kernel<true, true> : prep_tc_kernel<true, false>)
+                          : (one ? prep_tc_kernel<false, true> : prep_tc_kernel<false, false>);
+        e = opt_in_smem(kernel, sm, tc_opt_in[2 * bf + one]);
+        if (e != cudaSuccess) return e;
+        // after the statistics pass as a dependent launch; as the first kernel of the call in plain stream order
+        if (stats) e = launch_dependent(kernel, g2, PREP_THREADS, sm, stream, d_reqs, 0, h_reqs[0], dst);
+        else kernel<<<g2, PREP_THREADS, sm, stream>>>(d_reqs, 1, h_reqs[0], dst);
+    } else if (precision == FG21_PREC_FP32_DELTA) {
+        e = launch_dependent(prep_tiles_kernel<2>, g2, PREP_THREADS, sm, stream, d_reqs);
+    } else {
+        e = launch_dependent(prep_tiles_kernel<3>, g2, PREP_THREADS, sm, stream, d_reqs);
     }
     if (e != cudaSuccess) return e;
     return cudaGetLastError();

@@ -36,8 +36,10 @@ int num_sms_of(int device) {
 int Workspace::ensure(size_t dev_need, size_t arena_need, size_t pinned_need, int n_reqs) {
     if (device < 0) FG21_CUDA_TRY(cudaGetDevice(&device));
     if (!done) FG21_CUDA_TRY(cudaEventCreateWithFlags(&done, cudaEventDisableTiming));
-    // staging and scratch may still be in use by the previous call on this workspace
-    FG21_CUDA_TRY(cudaEventSynchronize(done));
+    // what is replaced or staged here may still be in use by the previous call on
+    // this workspace; otherwise a call follows it on the GPU alone (order_after)
+    if (dev_need > dev_bytes || arena_need > arena_bytes || pinned_need > 0 || n_reqs > reqs_cap)
+        FG21_CUDA_TRY(cudaEventSynchronize(done));
     if (!d_status) {
         void *p = nullptr;
         FG21_CUDA_TRY(cudaMalloc(&p, 256));
@@ -88,6 +90,23 @@ int Workspace::ensure(size_t dev_need, size_t arena_need, size_t pinned_need, in
     return FG21_OK;
 }
 
+// Orders `stream` after the workspace's previous call: a wait on its event
+// unless it was made on the same stream.  (Streams are told apart by their id,
+// which is never used twice, not by the handle.)
+int Workspace::order_after(cudaStream_t stream) {
+    // a call of this kind cannot be captured into a caller's graph: its workspace
+    // may be replaced by any later call
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    FG21_CUDA_TRY(cudaStreamIsCapturing(stream, &cap));
+    if (cap != cudaStreamCaptureStatusNone)
+        return set_error(FG21_E_CUDA, "the stream is being captured (fg21_graph_create captures an evaluation)");
+    unsigned long long id = 0;
+    FG21_CUDA_TRY(cudaStreamGetId(stream, &id));
+    if (called && id != last_stream) FG21_CUDA_TRY(cudaStreamWaitEvent(stream, done, 0));
+    last_stream = id;
+    return FG21_OK;
+}
+
 // The timing events are created when timing is switched on, never inside a
 // timed call (creating thousands of events takes milliseconds).
 int Workspace::timing_prepare() {
@@ -128,6 +147,7 @@ void Workspace::release() {
     d_status = nullptr;
     d_invalid = nullptr;
     done = nullptr;
+    called = false;
     dev_bytes = arena_bytes = pinned_bytes = 0;
     reqs_cap = 0;
 }
@@ -234,7 +254,8 @@ int prepare_requests(Workspace &ws, std::vector<ReqDesc> &reqs, int precision, P
         arena_need += lay[k].tiles;
         dev_need += lay[k].total() - lay[k].tiles;
     }
-    int rc = ws.ensure(dev_need, arena_need, sizeof(ReqDesc) * n, n);
+    // a single request's descriptor travels as a kernel argument, several are staged
+    int rc = ws.ensure(dev_need, arena_need, n > 1 ? sizeof(ReqDesc) * n : 0, n);
     if (rc) return rc;
     char *p = ws.dev;
     int64_t item = 0, row = 0, pts = 0;
@@ -293,7 +314,7 @@ int prepare_requests(Workspace &ws, std::vector<ReqDesc> &reqs, int precision, P
         L.alpha = false;
         for (int k = 0; k < n; ++k) L.alpha = L.alpha || reqs[k].Na > 0;
     }
-    std::memcpy(ws.pinned, reqs.data(), sizeof(ReqDesc) * n);
+    if (n > 1) std::memcpy(ws.pinned, reqs.data(), sizeof(ReqDesc) * n);
     return FG21_OK;
 }
 
@@ -301,13 +322,12 @@ int launch_requests(Workspace &ws, const std::vector<ReqDesc> &reqs, const Prepa
                     bool upload, bool timing) {
     const int n = pp.n;
     if (n == 0) return FG21_OK;
-    FG21_CUDA_TRY(cudaMemsetAsync(ws.d_status, 0, status_bytes(n), stream));   // status word, invalid counter
-    if (upload)
+    if (upload && n > 1)
         FG21_CUDA_TRY(cudaMemcpyAsync(ws.d_reqs, ws.pinned, sizeof(ReqDesc) * n, cudaMemcpyHostToDevice, stream));
     cudaEvent_t *ev = timing ? ws.timing_slot() : nullptr;
     if (ev) FG21_CUDA_TRY(cudaEventRecord(ev[0], stream));
     FG21_CUDA_TRY(launch_prep(reqs.data(), ws.d_reqs, n, pp.precision, pp.max_blocks, pp.max_fchunks, pp.max_tiles,
-                              stream));
+                              upload, stream));
     if (ev) FG21_CUDA_TRY(cudaEventRecord(ev[1], stream));
     if (pp.tc) {
         cudaError_t e = launch_tc(pp.tcl, pp.num_sms, stream);
@@ -325,9 +345,12 @@ int enqueue_requests(Workspace &ws, std::vector<ReqDesc> &reqs, int precision, c
     Prepared pp;
     int rc = prepare_requests(ws, reqs, precision, pp);
     if (rc || pp.n == 0) return rc;
+    rc = ws.order_after(stream);
+    if (rc) return rc;
     rc = launch_requests(ws, reqs, pp, stream, true, true);
     if (rc) return rc;
     FG21_CUDA_TRY(cudaEventRecord(ws.done, stream));
+    ws.called = true;
     return FG21_OK;
 }
 

@@ -26,6 +26,9 @@ struct Workspace {
     unsigned *d_status = nullptr;   // bytes 0..3 status word, 16..23 invalid counter
     unsigned long long *d_invalid = nullptr;
     cudaEvent_t done = nullptr;     // recorded after the last launch of a call
+    bool called = false;            // ... which there has been
+    unsigned long long last_stream = 0;   // id of that call's stream
+    int order_after(cudaStream_t stream);
     bool timing = false;            // record events around prep / main / reduce of every call
     static constexpr int TIMING_CAP = 8192;
     std::vector<cudaEvent_t> tev;   // [TIMING_CAP][4], created on first use
@@ -56,8 +59,8 @@ struct Prepared {
     TcLaunch tcl{};
 };
 int prepare_requests(Workspace &ws, std::vector<ReqDesc> &reqs, int precision, Prepared &pp);
-// ... and enqueue the status clear, the descriptor upload (if `upload`) and
-// the kernels.  Nothing here allocates or synchronises, so it can be captured
+// ... and enqueue the kernels, the descriptors stored first if `upload` (one as
+// a kernel argument, several by a copy).  Nothing here allocates or synchronises, so it can be captured
 // into a CUDA graph.
 int launch_requests(Workspace &ws, const std::vector<ReqDesc> &reqs, const Prepared &pp, cudaStream_t stream,
                     bool upload, bool timing);

@@ -13,9 +13,9 @@
 // until the process exits.  It runs the same kernels (prep, tensor-core
 // likelihood, reduction) as fg21_loglike_batch_device.
 //
-// The request descriptor reaches the array through the arguments of a
-// one-thread kernel (kernel arguments are copied when the launch is enqueued),
-// so no host buffer has to outlive the call.
+// The request descriptor reaches the array through the arguments of the first
+// kernel (kernel arguments are copied when the launch is enqueued), so no host
+// buffer has to outlive the call.
 //
 // Every call shares the array and leaves its contents behind: the status word
 // and invalid counter are cleared at the start of each call, everything else
@@ -59,10 +59,6 @@ int noalloc_base(int device, char **base) {
 }
 
 size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
-
-// Stores the request descriptor, passed by value, into the scratch array.
-static_assert(sizeof(ReqDesc) <= 4096, "the request descriptor travels as a kernel argument");
-__global__ void store_desc_kernel(const ReqDesc r, ReqDesc *dst) { *dst = r; }
 
 }  // namespace
 }  // namespace fg21
@@ -125,11 +121,8 @@ extern "C" int fg21_loglike_batch_device_noalloc(fg21_model *m, const double *d_
     r.status = status;
     r.invalid = reinterpret_cast<unsigned long long *>(base + 16);
 
-    // the status word and invalid counter start at zero; the rest is rewritten
-    FG21_CUDA_TRY(cudaMemsetAsync(status, 0, status_bytes(1), s));
-    store_desc_kernel<<<1, 1, 0, s>>>(r, d_req);
-    FG21_CUDA_TRY(cudaGetLastError());
-    FG21_CUDA_TRY(launch_prep(&r, d_req, 1, precision, r.n_stat_blocks, r.F * r.n_tchunks, r.n_tiles, s));
+    // prep stores the descriptor and zeroes the status word and invalid counter; the rest is rewritten
+    FG21_CUDA_TRY(launch_prep(&r, d_req, 1, precision, r.n_stat_blocks, r.F * r.n_tchunks, r.n_tiles, true, s));
     TcLaunch T;
     T.d_reqs = d_req;
     T.n_reqs = 1;
