@@ -460,7 +460,8 @@ __device__ __forceinline__ int64_t item_step() { return (int64_t)gridDim.x * LAN
 // 0 takes both at run time, for the forms that are not worth their own code.
 // ALPHA (amplitude regions): the series runs on y = d nL + g with g = ln(alpha
 // / abar) of each component; the coefficients 2^(-s j) / j! are then the same
-// for every channel.  DF: the series degree (3, 5 or 8).  With the short series
+// for every channel.  DF: the series degree (3, 5, 8, or 9: degree 8 of an
+// argument halved s >= 1 times, and as many squarings).  With the short series
 // (D = 3: a batch spread below ~0.007 in beta, as near a posterior) the
 // deviations' low parts enter the weights.
 template <int KP, bool BF16, int KR, int NEV, bool ALPHA, int DF>
@@ -470,6 +471,7 @@ __device__ __forceinline__ bool gen_item(const Params &prm, Barriers *S, uint32_
     constexpr int UNITS = (FIXED ? KR : KP) / 16;          // K steps of the row: 8 pairs each
     constexpr int NP = FIXED ? NEV * 4 : KP / 2;           // pairs that may hold regions
     constexpr bool LO = DF == 3 && !ALPHA;
+    constexpr int DEG = DF == 9 ? 8 : DF;
     constexpr bool X2 = LO || ALPHA;                       // a second operand per pair: the low part, or g
     constexpr bool X2_REGS = X2 && KP <= 32;               // ... kept in registers
     const int Kr = FIXED ? KR : uni(r.Kp), nch = uni(r.n_tchunks);
@@ -498,13 +500,13 @@ __device__ __forceinline__ bool gen_item(const Params &prm, Barriers *S, uint32_
     const float *__restrict__ nup = r.nu32;
     const float *__restrict__ nLp = r.nL32;
     const unsigned long long *__restrict__ coef = r.coef2;
-    uint64_t e2[DF + 1];
+    uint64_t e2[DEG + 1];
     e2[0] = 0;
     if (ALPHA) {
         const float ys = exp2i(-sp.s);
         float pw = sp.s ? 1.0f : sW, fact = 1.0f;
 #pragma unroll
-        for (int j = 1; j <= DF; ++j) {
+        for (int j = 1; j <= DEG; ++j) {
             pw *= ys;
             fact *= (float)j;
             const float e = pw * (1.0f / fact);
@@ -521,10 +523,10 @@ __device__ __forceinline__ bool gen_item(const Params &prm, Barriers *S, uint32_
             // the channel's coefficients e_j = (nL / 2^s)^j / j! (times 2^sW when s = 0), packed pairs
             const ulonglong2 *cf = reinterpret_cast<const ulonglong2 *>(coef + (size_t)f * 8);
 #pragma unroll
-            for (int j = 0; 2 * j < DF; ++j) {
+            for (int j = 0; 2 * j < DEG; ++j) {
                 const ulonglong2 v = __ldg(cf + j);
                 e2[2 * j + 1] = v.x;
-                if (2 * j + 2 <= DF) e2[2 * j + 2] = v.y;
+                if (2 * j + 2 <= DEG) e2[2 * j + 2] = v.y;
             }
         }
         const float s21 = a21 * __expf(-dnu * dnu * inv2s2);
@@ -558,8 +560,8 @@ __device__ __forceinline__ bool gen_item(const Params &prm, Barriers *S, uint32_
                         }
                         if (ALPHA) y2[i] = fma2(y2[i], nL2, l2[i]);
                     }
-                    em1_series2<DF, CH, LO>(w, y2, e2, l2);
-                    if (DF == 8 && !FIXED && sp.s > 0) {
+                    em1_series2<DEG, CH, LO>(w, y2, e2, l2);
+                    if (DF == 9) {
                         const uint64_t two2 = pk2(2.0f, 2.0f), sW2 = pk2(sW, sW);
                         for (int k = 0; k < sp.s; ++k)
 #pragma unroll
@@ -596,49 +598,49 @@ __device__ __forceinline__ bool gen_item_any(const Params &prm, Barriers *S, uin
     const SeriesPlan sp{uni(r.scaleW[1]), uni(r.scaleW[2])};
     return sp.D == 3 ? gen_item<KP, BF16, 0, 0, ALPHA, 3>(prm, S, stage, slot0, r, it, sp, w_lane, m)
          : sp.D == 5 ? gen_item<KP, BF16, 0, 0, ALPHA, 5>(prm, S, stage, slot0, r, it, sp, w_lane, m)
-                     : gen_item<KP, BF16, 0, 0, ALPHA, 8>(prm, S, stage, slot0, r, it, sp, w_lane, m);
+         : sp.s == 0 ? gen_item<KP, BF16, 0, 0, ALPHA, 8>(prm, S, stage, slot0, r, it, sp, w_lane, m)
+                     : gen_item<KP, BF16, 0, 0, ALPHA, 9>(prm, S, stage, slot0, r, it, sp, w_lane, m);
 }
 
 // One item by the code for its K and chunk count: NEV chunks of regions and
 // the trough pair make K = 8 (NEV + 1) for an odd NEV, and 8 NEV or 8 (NEV + 2)
 // for an even one.
-template <int KP, bool BF16, int NEV>
+template <int KP, bool BF16, int NEV, bool ALPHA>
 __device__ __forceinline__ bool gen_item_nev(const Params &prm, Barriers *S, uint32_t &stage, uint32_t slot0,
                                              const ReqDesc &r, const Item &it, SeriesPlan sp, uint32_t w_lane, int m) {
     constexpr int K0 = NEV % 2 ? 8 * (NEV + 1) : 8 * NEV, K1 = NEV % 2 == 0 && 8 * (NEV + 2) <= KP ? 8 * (NEV + 2) : K0;
     if (K1 != K0 && uni(r.Kp == K1))
-        return sp.D == 3 ? gen_item<KP, BF16, K1, NEV, false, 3>(prm, S, stage, slot0, r, it, sp, w_lane, m)
-             : sp.D == 5 ? gen_item<KP, BF16, K1, NEV, false, 5>(prm, S, stage, slot0, r, it, sp, w_lane, m)
-                         : gen_item<KP, BF16, K1, NEV, false, 8>(prm, S, stage, slot0, r, it, sp, w_lane, m);
-    return sp.D == 3 ? gen_item<KP, BF16, K0, NEV, false, 3>(prm, S, stage, slot0, r, it, sp, w_lane, m)
-         : sp.D == 5 ? gen_item<KP, BF16, K0, NEV, false, 5>(prm, S, stage, slot0, r, it, sp, w_lane, m)
-                     : gen_item<KP, BF16, K0, NEV, false, 8>(prm, S, stage, slot0, r, it, sp, w_lane, m);
+        return sp.D == 3 ? gen_item<KP, BF16, K1, NEV, ALPHA, 3>(prm, S, stage, slot0, r, it, sp, w_lane, m)
+             : sp.D == 5 ? gen_item<KP, BF16, K1, NEV, ALPHA, 5>(prm, S, stage, slot0, r, it, sp, w_lane, m)
+         : sp.s == 0 ? gen_item<KP, BF16, K1, NEV, ALPHA, 8>(prm, S, stage, slot0, r, it, sp, w_lane, m)
+                     : gen_item<KP, BF16, K1, NEV, ALPHA, 9>(prm, S, stage, slot0, r, it, sp, w_lane, m);
+    return sp.D == 3 ? gen_item<KP, BF16, K0, NEV, ALPHA, 3>(prm, S, stage, slot0, r, it, sp, w_lane, m)
+         : sp.D == 5 ? gen_item<KP, BF16, K0, NEV, ALPHA, 5>(prm, S, stage, slot0, r, it, sp, w_lane, m)
+     : sp.s == 0 ? gen_item<KP, BF16, K0, NEV, ALPHA, 8>(prm, S, stage, slot0, r, it, sp, w_lane, m)
+                 : gen_item<KP, BF16, K0, NEV, ALPHA, 9>(prm, S, stage, slot0, r, it, sp, w_lane, m);
 }
-// Arguments above 0.55 (squarings) take the run-time form.
-template <int KP, bool BF16, bool FIXED>
+template <int KP, bool BF16, bool FIXED, bool ALPHA>
 __device__ __forceinline__ bool gen_item_k(const Params &prm, Barriers *S, uint32_t &stage, uint32_t slot0,
                                            const ReqDesc &r, const Item &it, uint32_t w_lane, int m) {
     if constexpr (FIXED) {
         constexpr int MAX_NEV = KP / 8;
         const SeriesPlan sp{uni(r.scaleW[1]), uni(r.scaleW[2])};
-        if (sp.s == 0) {
 #define FG21_NEV(n) \
     case n:         \
-        if constexpr (n <= MAX_NEV) return gen_item_nev<KP, BF16, n>(prm, S, stage, slot0, r, it, sp, w_lane, m);
-            switch (uni((r.N + 7) / 8)) {
-                FG21_NEV(1)
-                FG21_NEV(2)
-                FG21_NEV(3)
-                FG21_NEV(4)
-                FG21_NEV(5)
-                FG21_NEV(6)
-                FG21_NEV(7)
-                FG21_NEV(8)
-            }
-#undef FG21_NEV
+        if constexpr (n <= MAX_NEV) return gen_item_nev<KP, BF16, n, ALPHA>(prm, S, stage, slot0, r, it, sp, w_lane, m);
+        switch (uni((r.N + 7) / 8)) {
+            FG21_NEV(1)
+            FG21_NEV(2)
+            FG21_NEV(3)
+            FG21_NEV(4)
+            FG21_NEV(5)
+            FG21_NEV(6)
+            FG21_NEV(7)
+            FG21_NEV(8)
         }
+#undef FG21_NEV
     }
-    return gen_item_any<KP, BF16, false>(prm, S, stage, slot0, r, it, w_lane, m);
+    return gen_item_any<KP, BF16, ALPHA>(prm, S, stage, slot0, r, it, w_lane, m);
 }
 
 // ------------------------------------------------------------- epilogue
@@ -915,8 +917,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         for (int64_t item = first_item(lane_id); item < prm.n_items && ok; item += item_step()) {
             const Item it = decode_item(reqs, prm.n_reqs, item);
             const ReqDesc &r = reqs[it.req];
-            if (ALPHA && r.Na) ok = gen_item_any<KP, BF16, true>(prm, S, stage, slot0, r, it, w_lane, m);
-            else ok = gen_item_k<KP, BF16, !BF16 && !RESID && !ALPHA>(prm, S, stage, slot0, r, it, w_lane, m);
+            if (ALPHA && r.Na) ok = gen_item_k<KP, BF16, !BF16 && !RESID && KP <= 32, true>(prm, S, stage, slot0, r, it, w_lane, m);
+            else ok = gen_item_k<KP, BF16, !BF16 && !RESID && !ALPHA, false>(prm, S, stage, slot0, r, it, w_lane, m);
         }
     } else if (warp < WARP_TMA) {
         // ========================================================= epilogue
