@@ -142,6 +142,9 @@ struct ReqLayout {
 // Shape decisions for one request (autotuned channel grouping).
 void plan_request(ReqDesc &r, int precision, int num_sms, int64_t total_tiles_in_launch);
 ReqLayout request_layout(const ReqDesc &r, int precision);
+// Channels per item by waves of single items: the split that sets the documented
+// point limit of the allocation-free call.
+int channels_per_wave_item(int64_t tiles, int F, int num_sms);
 
 // ------------------------------------------------------- kernel launchers
 // All enqueue on `stream` and return cudaError_t of the launch.

@@ -181,6 +181,31 @@ static int choose_channels_per_group(int64_t total_tiles, int F, int slots, int 
     return best_cpg;
 }
 
+// Channels per work item of the tensor kernel, whose CTAs (one per SM) work on
+// two items at once: a CTA with m of the items takes about m / 2 rounds of two
+// and, for an odd m, one alone, which is 1.26 times as fast a stage as a pair
+// (0.54 against 0.68 us at 24 regions, 100 bins); an item costs about two stages
+// besides its own.  A stage is a channel's t-chunk.  Measured against counting
+// waves of single items (16384 points, 301 channels: the same split):
+// 3001 points, 211 channels, two chunks 71 us a call from 78; 8192 points, 301
+// channels, amplitude regions 91 from 97; 4096 points, 151 channels 29.9 from 31.
+static int choose_channels_tc(int64_t tiles, int F, int n_tchunks, int num_sms) {
+    if (g_cpg_override() > 0) return std::min(F, g_cpg_override());
+    double best = 1e300;
+    int best_cpg = F;
+    for (int cpg = 1; cpg <= F; ++cpg) {
+        const int64_t items = tiles * ((F + cpg - 1) / cpg), m = (items + num_sms - 1) / num_sms;
+        const double cost = (1.26 * (double)(m / 2) + (double)(m % 2)) * (cpg * n_tchunks + 2.0);
+        if (cost < best - 1e-9) {
+            best = cost;
+            best_cpg = cpg;
+        }
+    }
+    return best_cpg;
+}
+
+int channels_per_wave_item(int64_t tiles, int F, int num_sms) { return choose_channels_per_group(tiles, F, num_sms); }
+
 void plan_request(ReqDesc &r, int precision, int num_sms, int64_t total_tiles) {
     r.Kp = round16(r.N + 2);
     r.pts_rows = precision == FG21_PREC_FP16X3 || precision == FG21_PREC_BF16X3 ? r.Kp + 4 + (r.Na ? r.Kp : 0) + r.Kp
@@ -198,7 +223,7 @@ void plan_request(ReqDesc &r, int precision, int num_sms, int64_t total_tiles) {
     if (r.cpg_hint > 0) {
         cpg = std::min(r.F, r.cpg_hint);
     } else if (tc) {
-        cpg = choose_channels_per_group(total_tiles, r.F, num_sms);
+        cpg = choose_channels_tc(total_tiles, r.F, r.n_tchunks, num_sms);
     } else {
         // SIMT blocks are not persistent: the waves are counted in the blocks
         // the GPU holds at once (at most 32 groups, the reduction's serial row)

@@ -87,10 +87,21 @@ extern "C" int fg21_loglike_batch_device_noalloc(fg21_model *m, const double *d_
 
     // plan and lay out exactly as the regular call does, then carve the array
     ReqDesc r = model_request(m, d_params, P, d_logL, precision);
-    plan_request(r, precision, num_sms_of(dev), (P + TILE_M - 1) / TILE_M);
-    const ReqLayout L = request_layout(r, precision);
+    const int sms = num_sms_of(dev), hint = r.cpg_hint;
+    const int64_t tiles = (P + TILE_M - 1) / TILE_M;
     const size_t head = a256(status_bytes(1)) + a256(sizeof(ReqDesc));      // status block + descriptor
-    const size_t need = head + (L.total() - L.tiles) + a256(L.tiles);
+    ReqLayout L;
+    auto scratch = [&](int cpg) {
+        r.cpg_hint = cpg;
+        plan_request(r, precision, sms, tiles);
+        L = request_layout(r, precision);
+        return head + (L.total() - L.tiles) + a256(L.tiles);
+    };
+    // the limit is that of the split by waves; the planner's split (or the tuned
+    // one) is used where its partial sums fit as well
+    const int wave = hint > 0 ? hint : channels_per_wave_item(tiles, r.F, sms);
+    const size_t need = scratch(wave);
+    if (need <= FG21_NOALLOC_SCRATCH_BYTES && hint <= 0 && scratch(0) > FG21_NOALLOC_SCRATCH_BYTES) scratch(wave);
     if (need > FG21_NOALLOC_SCRATCH_BYTES)
         return set_error(FG21_E_RANGE,
                          "request needs %zu scratch bytes, above the %zu-byte limit of the no-allocation call "
