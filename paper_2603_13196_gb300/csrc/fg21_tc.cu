@@ -428,6 +428,8 @@ struct Params {
     int64_t n_items;
     int b_stage_bytes;     // bytes of one operand-tile stage
     int acc_cols;          // tensor-memory columns of a lane's accumulator
+    int half_col;          // ... and the first of its second half: the same for every request of a launch, so
+                           // that the halves of two items with other column counts never overlap
     int ring_log2;         // a lane's stage slots (operand tile, weight block, barriers): 1, 2 or 4
     uint32_t tmem_cols;    // allocated tensor-memory columns
     unsigned *status;
@@ -743,11 +745,11 @@ __device__ __forceinline__ bool epi_item(const Params &prm, Barriers *S, uint32_
             return false;
         tc_fence_after();
         if constexpr (RESID) {
-            const int Tc = r.Tc, T = r.T, F = r.F, nblk = r.Tc_pad / 16;
+            const int Tc = r.Tc, T = r.T, F = r.F, nblk = r.Tc_pad / 16, hb = (nblk + 1) / 2;
             const int f = it.f0 + k / nch, t0 = (k % nch) * Tc, tn = min(Tc, T - t0);
             for (int b = 0; b < nblk; ++b) {
                 uint32_t v[16];
-                tmem_ld16(acc_lane + b * 16, v);
+                tmem_ld16(acc_lane + (b < hb ? b * 16 : prm.half_col + (b - hb) * 16), v);
                 tmem_ld_wait();
                 if (p < r.P)
 #pragma unroll
@@ -759,7 +761,7 @@ __device__ __forceinline__ bool epi_item(const Params &prm, Barriers *S, uint32_
             release(0);
             release(1);
         } else {
-            q1 = half_sumsq<NBLK - HB>(acc_lane + 16 * HB, [&] { release(1); });
+            q1 = half_sumsq<NBLK - HB>(acc_lane + prm.half_col, [&] { release(1); });
         }
         ++stage;
         qf0 += q0 * unscale * unscale;
@@ -841,7 +843,7 @@ __device__ __forceinline__ bool mma_item(const Params &prm, Barriers *S, uint32_
     const int n0 = (tc_pad / 16 + 1) / 2 * 16, n1 = tc_pad - n0;       // columns of the halves (n1 may be 0)
     const uint32_t idesc0 = instr_desc(128, n0, BF16), idesc1 = instr_desc(128, n1, BF16);
     const uint32_t b_lbo = (uint32_t)tc_pad * 16, b_split = 2 * KS * b_lbo;
-    const uint32_t d = tmem + (uint32_t)(lane_id * prm.acc_cols);
+    const uint32_t d = tmem + (uint32_t)(lane_id * prm.acc_cols), d1 = d + (uint32_t)prm.half_col;
     for (int k = 0; k < n; ++k) {
         const uint32_t slot = ((uint32_t)lane_id << prm.ring_log2) + slot_of(stage, prm.ring_log2);
         const uint32_t w_hi = tmem + w_col0 + slot * KP, b = b_slots + slot * prm.b_stage_bytes;
@@ -854,7 +856,7 @@ __device__ __forceinline__ bool mma_item(const Params &prm, Barriers *S, uint32_
         if (!mbar_wait(&S->acc_free[2 * lane_id + 1], (stage & 1u) ^ 1u, S, prm.status, STATUS_TIMEOUT_MMA))
             return false;
         tc_fence_after();
-        if (n1) issue_mmas<KS>(d + n0, w_hi, w_hi + 8 * KS, b + n0 * 16, b_lbo, b_split, idesc1, el);
+        if (n1) issue_mmas<KS>(d1, w_hi, w_hi + 8 * KS, b + n0 * 16, b_lbo, b_split, idesc1, el);
         mma_commit(&S->done[slot], el);
         ++stage;
     }
@@ -1063,6 +1065,7 @@ cudaError_t launch_common(const ReqDesc *d_reqs, int n_reqs, int64_t n_items, in
     prm.n_items = n_items;
     prm.b_stage_bytes = ((4 * kp_max * tc_pad_max) + 1023) & ~1023;
     prm.acc_cols = tc_pad_max;
+    prm.half_col = (tc_pad_max / 16 + 1) / 2 * 16;
     // Tensor memory, for each of the two lanes: an accumulator (used in halves),
     // and 4, 2 or 1 stage slots as the rest and shared memory (operand tiles,
     // barriers) hold.

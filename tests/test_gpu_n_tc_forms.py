@@ -38,3 +38,22 @@ def test_column_blocks(fg21lib, T):
 def test_items_over_lanes(fg21lib, tiles):
     # one channel: a work item per 128-point tile, so the lanes of 152 CTAs hold none, one or several
     _check(fg21lib, 3, 1, 2, [cases.I.prior_draws(128 * tiles - 5, 3, seed=tiles)])
+
+
+def test_items_of_other_widths_follow_each_other(fg21lib):
+    """Items with other numbers of columns, one after the other in a lane, use one
+    accumulator: what one still reads, the next must not write."""
+    models, params = [], []
+    for k, T in enumerate((10, 97, 33, 129, 1, 64, 177, 17, 80, 48)):
+        N = 3 + 4 * (k % 4)
+        sky, obs, m, data = cases.small_case(npix=1024, N=N, F=31, T=T, window=3.0)
+        model = fg21lib.fg21_build_regions(sky, obs, N)
+        fg21lib.fg21_model_set_data(model, data)
+        models.append(model)
+        params.append(cases.I.prior_draws(2500 - 130 * k, N, seed=k))
+    alone = [fg21lib.fg21_loglike_batch(m, p, "fp16x3") for m, p in zip(models, params)]
+    for rep in range(30):
+        order = np.random.default_rng(rep).permutation(len(models))
+        mixed = fg21lib.fg21_loglike_multi([models[i] for i in order], [params[i] for i in order], "fp16x3")
+        for i, got in zip(order, mixed):
+            assert np.array_equal(alone[i], got), (rep, models[i].T, int(np.sum(alone[i] != got)))
