@@ -12,10 +12,19 @@
 // to FP64 rounding; every sum is deterministic.
 //
 //   pass 1, one block per (f, t):   den[f,t] = sum_q num(q,f,t),  Bsum[f,t] = sum_q D(q,f,t)
+//           (B comes of it whatever the weighting)
 //   pass 2, one thread per (q, f):  pw[f,q]  = sum_t num(q,f,t) / den[f,t];
 //           one thread per q:       w[q]     = (1/(F T)) sum_f pw[f,q]
 //   pass 3, one block per (f, t):   A[c,f,t] = (1/Npix) sum_{q in component c} (T230_q - T_CMB) D(q,f,t)
 //           over the pixels sorted by component (contiguous segments).
+//
+// What bounds it is the FP64 exponential of D (this part's FP64 rate is 1/64 of
+// FP32's), needed by every pass: pass 1 keeps D [F][T][Npix] in device memory
+// where a quarter of what is free holds it (0.3 GB at 12288 pixels, 151 channels, 20
+// bins; 11.8 GB at 49152, 301, 100) and the others read it; without the room they
+// evaluate it again.  The tables of one build serve both its halves.
+// 12288 pixels, 9 regions, 151 channels, 20 bins: 4.06 ms a build from 8.00 (four
+// evaluations of D, and the tables made twice).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -35,6 +44,7 @@ struct DevObs {
     const double *beam_p;  // [F]
     const double *logcT;   // [T][npix] ln(z_t . v_q), -inf below the horizon
     const double *tskyT;   // [F][npix] T_sky(q, f) (sky and beam weightings)
+    const double *D;       // [F][T][npix] the beam where pass 1 kept it, else null
     int64_t npix;
     int F, T;
     double t_cmb;
@@ -43,6 +53,11 @@ struct DevObs {
 __device__ __forceinline__ double beam_d(double lc, double p) {
     if (lc == -INFINITY) return 0.0;
     return 2.0 * (p + 1.0) * (p == 0.0 ? 1.0 : exp(p * lc));
+}
+
+// D of pixel q at (f, t) = row ft
+__device__ __forceinline__ double beam_at(const DevObs &o, int ft, int64_t q, double lc, double p) {
+    return o.D ? o.D[(size_t)ft * o.npix + q] : beam_d(lc, p);
 }
 
 __device__ __forceinline__ double importance_num(const DevObs &o, int weighting, int64_t q, int f, double lc,
@@ -89,8 +104,9 @@ __global__ void tsky_kernel(const double *__restrict__ t230, const double *__res
     tskyT[i] = (t230[q] - t_cmb) * exp(-beta[q] * lognu[f]) + t_cmb;
 }
 
-__global__ void __launch_bounds__(BUILD_THREADS) den_kernel(DevObs o, int weighting, double *__restrict__ den,
-                                                            double *__restrict__ bsum) {
+// inv_den = 1 / den (0 for an empty sum); keep (optional): where to put D.
+__global__ void __launch_bounds__(BUILD_THREADS) den_kernel(DevObs o, int weighting, double *__restrict__ inv_den,
+                                                            double *__restrict__ bsum, double *__restrict__ keep) {
     __shared__ double sh[BUILD_THREADS];
     const int ft = blockIdx.x, f = ft / o.T, t = ft % o.T;
     const double p = o.beam_p[f];
@@ -98,14 +114,15 @@ __global__ void __launch_bounds__(BUILD_THREADS) den_kernel(DevObs o, int weight
     double a = 0.0, b = 0.0;
     for (int64_t q = threadIdx.x; q < o.npix; q += BUILD_THREADS) {
         const double lc = lc_row[q];
-        const double d = beam_d(lc, p);
+        const double d = beam_at(o, ft, q, lc, p);
+        if (keep) keep[(size_t)ft * o.npix + q] = d;
         a += importance_num(o, weighting, q, f, lc, d);
         b += d;
     }
     a = block_sum(a, sh);
     b = block_sum(b, sh);
     if (threadIdx.x == 0) {
-        den[ft] = a;
+        inv_den[ft] = a > 0.0 ? 1.0 / a : 0.0;
         bsum[ft] = b;
     }
 }
@@ -120,7 +137,7 @@ __global__ void __launch_bounds__(BUILD_THREADS) pw_kernel(DevObs o, int weighti
     double acc = 0.0;
     for (int t = 0; t < o.T; ++t) {
         const double lc = o.logcT[(size_t)t * o.npix + q];
-        acc += importance_num(o, weighting, q, f, lc, beam_d(lc, p)) * inv_den[(size_t)f * o.T + t];
+        acc += importance_num(o, weighting, q, f, lc, beam_at(o, f * o.T + t, q, lc, p)) * inv_den[(size_t)f * o.T + t];
     }
     pw[(size_t)f * o.npix + q] = acc;
 }
@@ -146,72 +163,11 @@ __global__ void __launch_bounds__(BUILD_THREADS) resp_kernel(DevObs o, const dou
         double a = 0.0;
         for (int64_t k = seg[c] + threadIdx.x; k < seg[c + 1]; k += BUILD_THREADS) {
             const int64_t q = perm[k];
-            a += (t230[q] - o.t_cmb) * beam_d(lc_row[q], p);
+            a += (t230[q] - o.t_cmb) * beam_at(o, ft, q, lc_row[q], p);
         }
         a = block_sum(a, sh);
         if (threadIdx.x == 0) A[((size_t)c * o.F + f) * o.T + t] = a * inv;
     }
-}
-
-// Device copies of the inputs and the geometry tables, freed on destruction.
-struct DevBuild {
-    double *dirs = nullptr, *t230 = nullptr, *beta = nullptr, *lognu = nullptr, *beam_p = nullptr, *zen = nullptr;
-    double *logcT = nullptr, *tskyT = nullptr;
-    std::vector<void *> extra;
-    ~DevBuild() {
-        void *ps[] = {dirs, t230, beta, lognu, beam_p, zen, logcT, tskyT};
-        for (void *p : ps)
-            if (p) cudaFree(p);
-        for (void *p : extra) cudaFree(p);
-    }
-    template <typename T>
-    cudaError_t alloc(T **p, size_t n) {
-        cudaError_t e = cudaMalloc((void **)p, sizeof(T) * n);
-        if (e == cudaSuccess) extra.push_back(*p);
-        return e;
-    }
-};
-
-cudaError_t upload(double **dst, const double *src, size_t n) {
-    cudaError_t e = cudaMalloc((void **)dst, sizeof(double) * n);
-    if (e == cudaSuccess) e = cudaMemcpy(*dst, src, sizeof(double) * n, cudaMemcpyHostToDevice);
-    return e;
-}
-
-// inputs, ln c per (t, q) and (when needed) T_sky per (f, q)
-cudaError_t prepare(const fg21_sky *s, const fg21_obs *o, bool need_tsky, DevBuild &d, DevObs &g) {
-    const int64_t npix = s->npix;
-    const int F = o->F, T = o->T;
-    std::vector<double> lognu(F);
-    for (int f = 0; f < F; ++f) lognu[f] = std::log(o->nu[f] / o->nu0);
-    cudaError_t e = upload(&d.dirs, s->dirs, 3 * (size_t)npix);
-    if (e == cudaSuccess) e = upload(&d.t230, s->t230, npix);
-    if (e == cudaSuccess) e = upload(&d.beta, s->beta, npix);
-    if (e == cudaSuccess) e = upload(&d.lognu, lognu.data(), F);
-    if (e == cudaSuccess) e = upload(&d.beam_p, o->beam_p, F);
-    if (e == cudaSuccess) e = upload(&d.zen, o->zenith, 3 * (size_t)T);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&d.logcT, sizeof(double) * (size_t)npix * T);
-    if (e != cudaSuccess) return e;
-    const int th = BUILD_THREADS;
-    logc_kernel<<<(unsigned)((npix * T + th - 1) / th), th>>>(d.dirs, d.zen, npix, T, d.logcT);
-    e = cudaGetLastError();
-    if (e == cudaSuccess && need_tsky) {
-        e = cudaMalloc((void **)&d.tskyT, sizeof(double) * (size_t)npix * F);
-        if (e == cudaSuccess) {
-            tsky_kernel<<<(unsigned)((npix * F + th - 1) / th), th>>>(d.t230, d.beta, d.lognu, o->t_cmb, npix, F,
-                                                                     d.tskyT);
-            e = cudaGetLastError();
-        }
-    }
-    g.lognu = d.lognu;
-    g.beam_p = d.beam_p;
-    g.logcT = d.logcT;
-    g.tskyT = d.tskyT;
-    g.npix = npix;
-    g.F = F;
-    g.T = T;
-    g.t_cmb = o->t_cmb;
-    return e;
 }
 
 int fail(cudaError_t e, const char *what) {
@@ -222,52 +178,130 @@ int fail(cudaError_t e, const char *what) {
 
 }  // namespace
 
-int device_importance(const fg21_sky *s, const fg21_obs *o, int weighting, std::vector<double> &w,
-                      std::vector<double> *B) {
-    DevBuild d;
+// Device copies of the inputs, the geometry tables and the beam of one build,
+// freed on destruction.
+struct DeviceBuild {
+    const fg21_sky *s;
+    const fg21_obs *o;
     DevObs g{};
-    const bool need_tsky = weighting == FG21_WEIGHT_BEAM || weighting == FG21_WEIGHT_SKY;
-    cudaError_t e = prepare(s, o, need_tsky, d, g);
-    if (e != cudaSuccess) return fail(e, "region building (inputs)");
+    double *t230 = nullptr, *beta = nullptr, *lognu = nullptr, *tsky = nullptr, *beam = nullptr;
+    double *inv_den = nullptr, *bsum = nullptr;
+    bool ready = false, summed = false;      // tables made; bsum (and beam) written
+    std::vector<void *> own;
+    ~DeviceBuild() {
+        for (void *p : own) cudaFree(p);
+    }
+    template <typename T>
+    cudaError_t alloc(T **p, size_t n) {
+        cudaError_t e = cudaMalloc((void **)p, sizeof(T) * n);
+        if (e == cudaSuccess) own.push_back(*p);
+        return e;
+    }
+    cudaError_t prepare(bool need_tsky);
+    cudaError_t pass1(int weighting);
+};
+
+namespace {
+cudaError_t upload(std::vector<void *> &own, double **dst, const double *src, size_t n) {
+    cudaError_t e = cudaMalloc((void **)dst, sizeof(double) * n);
+    if (e != cudaSuccess) return e;
+    own.push_back(*dst);
+    return cudaMemcpy(*dst, src, sizeof(double) * n, cudaMemcpyHostToDevice);
+}
+}  // namespace
+
+// inputs, ln c per (t, q) and (when needed) T_sky per (f, q)
+cudaError_t DeviceBuild::prepare(bool need_tsky) {
     const int64_t npix = s->npix;
-    const int F = o->F, T = o->T;
-    double *den = nullptr, *bsum = nullptr, *pw = nullptr, *dw = nullptr;
-    e = d.alloc(&den, (size_t)F * T);
-    if (e == cudaSuccess) e = d.alloc(&bsum, (size_t)F * T);
-    if (e == cudaSuccess) e = d.alloc(&pw, (size_t)F * npix);
-    if (e == cudaSuccess) e = d.alloc(&dw, (size_t)npix);
+    const int F = o->F, T = o->T, th = BUILD_THREADS;
+    cudaError_t e = cudaSuccess;
+    if (!ready) {
+        std::vector<double> ln(F);
+        for (int f = 0; f < F; ++f) ln[f] = std::log(o->nu[f] / o->nu0);
+        double *dirs = nullptr, *zen = nullptr, *beam_p = nullptr, *logcT = nullptr;
+        e = upload(own, &dirs, s->dirs, 3 * (size_t)npix);
+        if (e == cudaSuccess) e = upload(own, &t230, s->t230, npix);
+        if (e == cudaSuccess) e = upload(own, &beta, s->beta, npix);
+        if (e == cudaSuccess) e = upload(own, &lognu, ln.data(), F);
+        if (e == cudaSuccess) e = upload(own, &beam_p, o->beam_p, F);
+        if (e == cudaSuccess) e = upload(own, &zen, o->zenith, 3 * (size_t)T);
+        if (e == cudaSuccess) e = alloc(&logcT, (size_t)npix * T);
+        if (e == cudaSuccess) e = alloc(&inv_den, (size_t)F * T);
+        if (e == cudaSuccess) e = alloc(&bsum, (size_t)F * T);
+        if (e != cudaSuccess) return e;
+        logc_kernel<<<(unsigned)((npix * T + th - 1) / th), th>>>(dirs, zen, npix, T, logcT);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        g.lognu = lognu;
+        g.beam_p = beam_p;
+        g.logcT = logcT;
+        g.npix = npix;
+        g.F = F;
+        g.T = T;
+        g.t_cmb = o->t_cmb;
+        // room for the beam: at most a quarter of the free memory, and no error without it
+        const size_t need = sizeof(double) * (size_t)npix * F * T;
+        size_t free_bytes = 0, total = 0;
+        if (cudaMemGetInfo(&free_bytes, &total) == cudaSuccess && need <= free_bytes / 4 &&
+            alloc(&beam, (size_t)npix * F * T) != cudaSuccess)
+            beam = nullptr;
+        cudaGetLastError();
+        ready = true;
+    }
+    if (need_tsky && !tsky) {
+        e = alloc(&tsky, (size_t)npix * F);
+        if (e != cudaSuccess) return e;
+        tsky_kernel<<<(unsigned)((npix * F + th - 1) / th), th>>>(t230, beta, lognu, o->t_cmb, npix, F, tsky);
+        e = cudaGetLastError();
+        g.tskyT = tsky;
+    }
+    return e;
+}
+
+cudaError_t DeviceBuild::pass1(int weighting) {
+    den_kernel<<<(unsigned)(g.F * g.T), BUILD_THREADS>>>(g, weighting, inv_den, bsum, summed ? nullptr : beam);
+    const cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess && !summed) {
+        g.D = beam;
+        summed = true;
+    }
+    return e;
+}
+
+DeviceBuild *device_build_begin(const fg21_sky *s, const fg21_obs *o) {
+    DeviceBuild *b = new DeviceBuild;
+    b->s = s;
+    b->o = o;
+    return b;
+}
+void device_build_end(DeviceBuild *b) { delete b; }
+
+int device_importance(DeviceBuild *b, int weighting, std::vector<double> &w) {
+    const bool need_tsky = weighting == FG21_WEIGHT_BEAM || weighting == FG21_WEIGHT_SKY;
+    cudaError_t e = b->prepare(need_tsky);
+    if (e != cudaSuccess) return fail(e, "region building (inputs)");
+    const int64_t npix = b->g.npix;
+    const int F = b->g.F, T = b->g.T, th = BUILD_THREADS;
+    double *pw = nullptr, *dw = nullptr;
+    e = b->alloc(&pw, (size_t)F * npix);
+    if (e == cudaSuccess) e = b->alloc(&dw, (size_t)npix);
     if (e != cudaSuccess) return fail(e, "region building (importance)");
-    den_kernel<<<(unsigned)(F * T), BUILD_THREADS>>>(g, weighting, den, bsum);
-    if ((e = cudaGetLastError()) != cudaSuccess) return fail(e, "den_kernel");
-    std::vector<double> h_den((size_t)F * T), h_b((size_t)F * T);
-    if ((e = cudaMemcpy(h_den.data(), den, sizeof(double) * F * T, cudaMemcpyDeviceToHost)) != cudaSuccess ||
-        (e = cudaMemcpy(h_b.data(), bsum, sizeof(double) * F * T, cudaMemcpyDeviceToHost)) != cudaSuccess)
-        return fail(e, "region building (den)");
-    for (auto &x : h_den) x = x > 0.0 ? 1.0 / x : 0.0;
-    if ((e = cudaMemcpy(den, h_den.data(), sizeof(double) * F * T, cudaMemcpyHostToDevice)) != cudaSuccess)
-        return fail(e, "region building (1/den)");
-    const int th = BUILD_THREADS;
-    pw_kernel<<<dim3((unsigned)((npix + th - 1) / th), (unsigned)F), th>>>(g, weighting, den, pw);
+    if ((e = b->pass1(weighting)) != cudaSuccess) return fail(e, "den_kernel");
+    pw_kernel<<<dim3((unsigned)((npix + th - 1) / th), (unsigned)F), th>>>(b->g, weighting, b->inv_den, pw);
     w_kernel<<<(unsigned)((npix + th - 1) / th), th>>>(pw, npix, F, 1.0 / ((double)F * (double)T), dw);
     if ((e = cudaGetLastError()) != cudaSuccess) return fail(e, "w_kernel");
     w.resize(npix);
     if ((e = cudaMemcpy(w.data(), dw, sizeof(double) * npix, cudaMemcpyDeviceToHost)) != cudaSuccess)
         return fail(e, "region building (w)");
-    if (B) {
-        B->resize((size_t)F * T);
-        for (size_t k = 0; k < h_b.size(); ++k) (*B)[k] = h_b[k] / (double)npix;
-    }
     return FG21_OK;
 }
 
-int device_precompute(const fg21_sky *s, const fg21_obs *o, const std::vector<int32_t> &lab, int N,
-                      std::vector<double> &A, std::vector<double> &B) {
-    DevBuild d;
-    DevObs g{};
-    cudaError_t e = prepare(s, o, false, d, g);
+int device_precompute(DeviceBuild *b, const std::vector<int32_t> &lab, int N, std::vector<double> &A,
+                      std::vector<double> &B) {
+    cudaError_t e = b->prepare(false);
     if (e != cudaSuccess) return fail(e, "region building (inputs)");
-    const int64_t npix = s->npix;
-    const int F = o->F, T = o->T;
+    const int64_t npix = b->g.npix;
+    const int F = b->g.F, T = b->g.T;
     // pixels of each component contiguous, in index order within a component
     std::vector<int64_t> seg(N + 1, 0), perm(npix);
     for (int64_t q = 0; q < npix; ++q) seg[lab[q] + 1]++;
@@ -277,23 +311,21 @@ int device_precompute(const fg21_sky *s, const fg21_obs *o, const std::vector<in
         for (int64_t q = 0; q < npix; ++q) perm[pos[lab[q]]++] = q;
     }
     int64_t *dperm = nullptr, *dseg = nullptr;
-    double *dA = nullptr, *den = nullptr, *bsum = nullptr;
-    e = d.alloc(&dperm, (size_t)npix);
-    if (e == cudaSuccess) e = d.alloc(&dseg, (size_t)N + 1);
-    if (e == cudaSuccess) e = d.alloc(&dA, (size_t)N * F * T);
-    if (e == cudaSuccess) e = d.alloc(&den, (size_t)F * T);
-    if (e == cudaSuccess) e = d.alloc(&bsum, (size_t)F * T);
+    double *dA = nullptr;
+    e = b->alloc(&dperm, (size_t)npix);
+    if (e == cudaSuccess) e = b->alloc(&dseg, (size_t)N + 1);
+    if (e == cudaSuccess) e = b->alloc(&dA, (size_t)N * F * T);
     if (e == cudaSuccess) e = cudaMemcpy(dperm, perm.data(), sizeof(int64_t) * npix, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(dseg, seg.data(), sizeof(int64_t) * (N + 1), cudaMemcpyHostToDevice);
+    // B = (1/Npix) sum_q D: pass 1 of the importance gave it
+    if (e == cudaSuccess && !b->summed) e = b->pass1(FG21_WEIGHT_UNIFORM);
     if (e != cudaSuccess) return fail(e, "region building (precompute)");
-    resp_kernel<<<(unsigned)(F * T), BUILD_THREADS>>>(g, d.t230, dperm, dseg, N, dA);
-    // B = (1/Npix) sum_q D: the uniform weighting's pass 1 gives it without T_sky
-    den_kernel<<<(unsigned)(F * T), BUILD_THREADS>>>(g, FG21_WEIGHT_UNIFORM, den, bsum);
+    resp_kernel<<<(unsigned)(F * T), BUILD_THREADS>>>(b->g, b->t230, dperm, dseg, N, dA);
     if ((e = cudaGetLastError()) != cudaSuccess) return fail(e, "resp_kernel");
     A.resize((size_t)N * F * T);
     B.resize((size_t)F * T);
     if ((e = cudaMemcpy(A.data(), dA, sizeof(double) * A.size(), cudaMemcpyDeviceToHost)) != cudaSuccess ||
-        (e = cudaMemcpy(B.data(), bsum, sizeof(double) * B.size(), cudaMemcpyDeviceToHost)) != cudaSuccess)
+        (e = cudaMemcpy(B.data(), b->bsum, sizeof(double) * B.size(), cudaMemcpyDeviceToHost)) != cudaSuccess)
         return fail(e, "region building (A, B)");
     for (auto &x : B) x /= (double)npix;
     return FG21_OK;

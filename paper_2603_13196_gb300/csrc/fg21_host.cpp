@@ -4,6 +4,7 @@
 // in the CUDA kernels of fg21_kernels.cu / fg21_tc.cu; nothing here evaluates
 // a likelihood on the CPU.
 #include <algorithm>
+#include <memory>
 #include <queue>
 #include <cmath>
 #include <cstdarg>
@@ -405,9 +406,11 @@ int build_host(const fg21_sky *sky, const fg21_obs *obs, const fg21_partition_op
     const int N = std::max(Na, 1) * Nb;
     try {
         Geometry g;
+        std::unique_ptr<DeviceBuild, void (*)(DeviceBuild *)> dev(device ? device_build_begin(sky, obs) : nullptr,
+                                                                  device_build_end);
         if (!device) build_geometry(sky, obs, g);
         auto weights = [&](int weighting, std::vector<double> &w) -> int {
-            if (device) return device_importance(sky, obs, weighting, w, nullptr);
+            if (device) return device_importance(dev.get(), weighting, w);
             importance(sky, obs, g, weighting, w);
             return FG21_OK;
         };
@@ -423,7 +426,7 @@ int build_host(const fg21_sky *sky, const fg21_obs *obs, const fg21_partition_op
             for (int64_t q = 0; q < sky->npix; ++q) comp[q] = out.lab_a[q] * Nb + out.lab[q];
         }
         if (device) {
-            if ((rc = device_precompute(sky, obs, comp, N, out.A, out.B))) return rc;
+            if ((rc = device_precompute(dev.get(), comp, N, out.A, out.B))) return rc;
         } else {
             precompute(sky, obs, g, comp, N, out.A, out.B);
         }

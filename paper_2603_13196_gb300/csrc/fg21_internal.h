@@ -197,14 +197,16 @@ cudaError_t launch_mma_probe(const uint16_t *a, const uint16_t *b, const float *
 int tc_box_rows(const int64_t *tile_rows, int n);
 int tc_map_init();  // resolves cuTensorMapEncodeTiled; FG21_OK or error
 
-// Region building on the current device (fg21_build.cu): the importance
-// weights w[npix] of `weighting` (Sec. 4.2) and, optionally, B[F][T]; the
-// response functions A[N][F][T] of the components `lab` (Sec. 2.2 eq.
-// chromatic_function) and B.  Same FP64 arithmetic as the host code, other
-// summation order.  FG21_OK or an error code (message set).
-int device_importance(const fg21_sky *s, const fg21_obs *o, int weighting, std::vector<double> &w,
-                      std::vector<double> *B);
-int device_precompute(const fg21_sky *s, const fg21_obs *o, const std::vector<int32_t> &lab, int N,
-                      std::vector<double> &A, std::vector<double> &B);
+// Region building on the current device (fg21_build.cu), the tables of one
+// build shared by its halves: the importance weights w[npix] of `weighting`
+// (Sec. 4.2), and the response functions A[N][F][T] of the components `lab`
+// (Sec. 2.2 eq. chromatic_function) with B[F][T].  Same FP64 arithmetic as the
+// host code, other summation order.  FG21_OK or an error code (message set).
+struct DeviceBuild;
+DeviceBuild *device_build_begin(const fg21_sky *s, const fg21_obs *o);
+void device_build_end(DeviceBuild *b);
+int device_importance(DeviceBuild *b, int weighting, std::vector<double> &w);
+int device_precompute(DeviceBuild *b, const std::vector<int32_t> &lab, int N, std::vector<double> &A,
+                      std::vector<double> &B);
 
 }  // namespace fg21
