@@ -1136,41 +1136,43 @@ __global__ void __launch_bounds__(REDUCE_THREADS) reduce_kernel(const ReqDesc *_
     const int64_t p = gid - r.pt_begin;
     if (p < 0 || p >= r.P) return;       // uniform over a warp in WARP mode
     if ((r.n_part > REDUCE_SERIAL_MAX) != WARP) return;
-    if (*r.status) {         // a kernel of this launch stopped early: its partials are incomplete
-        if (lane == 0) r.logL[p] = __longlong_as_double(0x7FF8000000000000ll);
-        return;
-    }
-    if (!r.pvalid[p]) {      // the statistics pass tested the point (point_valid)
-        if (lane == 0) {
-            r.logL[p] = -INFINITY;
-            atomicAdd(r.invalid, 1ull);
-        }
-        return;
-    }
+    // everything a point reads is asked for before the first of it is looked at:
+    // the kernel is a chain of L2 latencies (4096 points, rows of 18 partials: 28.7 us
+    // a call from 29.3 with four loads in flight and the tests first)
+    const unsigned status = *r.status;
+    const unsigned char valid = r.pvalid[p];       // the statistics pass tested the point (point_valid)
+    const double2 nm = r.pnorm ? r.pnorm[p] : make_double2(0.0, 0.0);
     float sh = 0.0f, sl = 0.0f;
     const float2 *__restrict__ part = r.partials + (size_t)p * r.n_part;
-    if (WARP) {
-        for (int g = lane; g < r.n_part; g += 32) {
-            const float2 v = part[g];
-            two_sum_acc(sh, sl, v.x);
-            two_sum_acc(sh, sl, v.y);
-        }
+    constexpr int UN = WARP ? 4 : 16, STEP = WARP ? 32 : 1;
+    for (int g0 = lane; g0 < r.n_part; g0 += UN * STEP) {
+        float2 v[UN];
+#pragma unroll
+        for (int u = 0; u < UN; ++u) v[u] = g0 + u * STEP < r.n_part ? part[g0 + u * STEP] : make_float2(0.0f, 0.0f);
+#pragma unroll
+        for (int u = 0; u < UN; ++u)
+            if (g0 + u * STEP < r.n_part) {
+                two_sum_acc(sh, sl, v[u].x);
+                two_sum_acc(sh, sl, v[u].y);
+            }
+    }
+    if (WARP)
         for (int o = 16; o > 0; o >>= 1) {
             const float oh = __shfl_xor_sync(0xffffffffu, sh, o), ol = __shfl_xor_sync(0xffffffffu, sl, o);
             df_add(sh, sl, oh, ol);
         }
-        if (lane != 0) return;
-    } else {
-#pragma unroll 4
-        for (int g = 0; g < r.n_part; ++g) {
-            const float2 v = part[g];
-            two_sum_acc(sh, sl, v.x);
-            two_sum_acc(sh, sl, v.y);
-        }
+    if (lane != 0) return;
+    if (status) {            // a kernel of this launch stopped early: its partials are incomplete
+        r.logL[p] = __longlong_as_double(0x7FF8000000000000ll);
+        return;
+    }
+    if (!valid) {
+        r.logL[p] = -INFINITY;
+        atomicAdd(r.invalid, 1ull);
+        return;
     }
     const double chi2 = ((double)sh + (double)sl) * r.chi2_scale;
     if (r.pnorm) {           // sigma_n terms from prep (tensor path)
-        const double2 nm = r.pnorm[p];
         r.logL[p] = -0.5 * (nm.x + chi2 * nm.y);
     } else {
         const double sig = r.params[p * (r.NPF + 4) + r.NPF + 3];
