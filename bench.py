@@ -637,7 +637,7 @@ def noise_phase(fg21, stream, reps, n_cells, K=65536, sigma=0.025):
 def small_batch_phase(fg21, I, stream, K=200):
     """The launch-latency-bound end of the workloads: 64 prior draws at N = 3,
     F = 151, T = 1 (3072-pixel sky, hierarchical regions).  Median time per
-    evaluation of the direct device call (plan, descriptor upload, four launches),
+    evaluation of the direct device call (plan and launches),
     of the graph replay, and of the host-buffer call on page-locked buffers."""
     import numpy as np
     import torch
@@ -876,7 +876,7 @@ def main():
         "config": {"workload": WORKLOAD, "N": N, "F": F, "T": T, "P_per_gpu": P, "npix": wl.npix,
                    "precision": args.precision, "parallelism": f"replicas x{ws}",
                    "channels_per_item": cpg, "channels_per_item_from": "fg21_autotune (measured)",
-                   "path": "fg21_graph_launch: the step (status clear, prep, tensor-core, reduce kernels) "
+                   "path": "fg21_graph_launch: the step (prep, tensor-core, reduce kernels) "
                            "replayed from a CUDA graph captured once on the device buffers",
                    "l2": "flushed by a 256 MiB write between timed steps (not timed)",
                    "build_regions_s": round(build_s, 3)},
@@ -890,8 +890,8 @@ def main():
                                                    "median SM clock sampled during the timed region"}},
         "kernels_ms": {"prep": res["prep_ms"], "tc_loglike": res["main_ms"], "reduce": res["reduce_ms"]},
         "direct_call": {"value": P * ws / (call_ms * 1e-3), "unit": "logL evals/s", "ms_per_step": call_ms,
-                        "what": "the same step through fg21_loglike_batch_device each time (plan, descriptor "
-                                "upload and four launches per call)"},
+                        "what": "the same step through fg21_loglike_batch_device each time (plan "
+                                "and launches per call)"},
         "near_posterior": {"value": replica_throughput(P, ws, near_ms), "unit": "logL evals/s", "ms_per_step": near_ms,
                            "what": "the graph-replayed step on 16384 points within 1e-5 in beta of one point, "
                                    "as a nested sampler's late batches are (L2 flushed between steps)"},
