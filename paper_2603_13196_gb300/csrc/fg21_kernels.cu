@@ -226,7 +226,7 @@ __device__ __forceinline__ void gather_stats(const ReqDesc &r, float *sh /* [2 N
         for (int b0 = g; b0 < nb; b0 += 16 * G) {
             float x[16];
 #pragma unroll
-            for (int u = 0; u < 16; ++u) x[u] = b0 + u * G < nb ? __ldg(q + (size_t)(b0 + u * G) * W) : 0.0f;
+            for (int u = 0; u < 16; ++u) x[u] = b0 + u * G < nb ? q[(size_t)(b0 + u * G) * W] : 0.0f;
 #pragma unroll
             for (int u = 0; u < 16; ++u)
                 if (b0 + u * G < nb) v = kind == 0 ? v + x[u] : kind == 1 ? fminf(v, x[u]) : fmaxf(v, x[u]);
@@ -347,7 +347,7 @@ static_assert(sizeof(ReqDesc) % 8 == 0 && sizeof(ReqDesc) <= 2048, "the descript
 // ONE: the launch's only request, passed by value (stored at `store` unless
 // null); otherwise reqs[blockIdx.y].
 template <bool ONE>
-__global__ void __launch_bounds__(STAT_BLOCK) prep_stats_kernel(const ReqDesc *__restrict__ reqs, int staged,
+__global__ void __launch_bounds__(STAT_BLOCK) prep_stats_kernel(const ReqDesc *reqs, int staged,
                                                                 const __grid_constant__ ReqDesc one, ReqDesc *store) {
     // shared: [STAT_BLOCK / 32][2 NPF + 2] FP32 warp partials, then (staged) the
     // block's parameter rows [STAT_BLOCK][padded_row(NPF + 4)] FP64
@@ -504,7 +504,7 @@ __device__ __forceinline__ void prep_points(const ReqDesc &r, int tile, const do
 // or their deviations beta - bbar (delta form), then the amplitudes (direct) or
 // ln(alpha / abar) (delta).
 template <int MODE>  // 2 = SIMT delta, 3 = SIMT direct
-__global__ void __launch_bounds__(PREP_THREADS) prep_tiles_kernel(const ReqDesc *__restrict__ reqs) {
+__global__ void __launch_bounds__(PREP_THREADS) prep_tiles_kernel(const ReqDesc *reqs) {
     extern __shared__ double smem_d[];
     pdl_wait();
     const ReqDesc &r = reqs[blockIdx.y];
@@ -602,7 +602,7 @@ __global__ void __launch_bounds__(PREP_THREADS) prep_tiles_kernel(const ReqDesc 
 // [Tc_pad], wbar hi / lo [N] (FP32); points: parameter rows
 // [128][padded_row(NPF+4)] FP64.
 template <bool BF16, bool ONE>
-__global__ void __launch_bounds__(PREP_THREADS) prep_tc_kernel(const ReqDesc *__restrict__ reqs, int begin,
+__global__ void __launch_bounds__(PREP_THREADS) prep_tc_kernel(const ReqDesc *reqs, int begin,
                                                                const __grid_constant__ ReqDesc one, ReqDesc *store) {
     extern __shared__ double smem_d[];
     __shared__ float sh_red[PREP_THREADS / 32];
@@ -811,7 +811,7 @@ __device__ __forceinline__ void kahan_add(float &s, float &c, float x) {
     s = t;
 }
 
-__device__ __forceinline__ int find_req_by_item(const ReqDesc *__restrict__ reqs, int n_reqs, int64_t item) {
+__device__ __forceinline__ int find_req_by_item(const ReqDesc *reqs, int n_reqs, int64_t item) {
     int lo = 0, hi = n_reqs - 1;
     while (lo < hi) {
         int mid = (lo + hi + 1) >> 1;
@@ -820,7 +820,7 @@ __device__ __forceinline__ int find_req_by_item(const ReqDesc *__restrict__ reqs
     return lo;
 }
 
-__device__ __forceinline__ int find_req_by_point(const ReqDesc *__restrict__ reqs, int n_reqs, int64_t pt) {
+__device__ __forceinline__ int find_req_by_point(const ReqDesc *reqs, int n_reqs, int64_t pt) {
     int lo = 0, hi = n_reqs - 1;
     while (lo < hi) {
         int mid = (lo + hi + 1) >> 1;
@@ -842,7 +842,7 @@ __host__ __device__ inline size_t simt_smem_floats(int N, int tc) {
 constexpr size_t SIMT_SMEM_MAX = 226 * 1024;      // bytes a block may take (227 KB less the driver's share)
 
 template <bool DIRECT>
-__global__ void __launch_bounds__(SIMT_THREADS) simt_kernel(const ReqDesc *__restrict__ reqs, int n_reqs) {
+__global__ void __launch_bounds__(SIMT_THREADS) simt_kernel(const ReqDesc *reqs, int n_reqs) {
     extern __shared__ __align__(16) float smem_f[];
     pdl_wait();
     const int64_t item = blockIdx.x;
@@ -859,7 +859,7 @@ __global__ void __launch_bounds__(SIMT_THREADS) simt_kernel(const ReqDesc *__res
     float *qp = s21s + TILE_M;                        // [SIMT_CS + 1][128] per-slot point sums
     const int tid = threadIdx.x;
     // this point's parameter rows: [Nb] beta (plain) or beta - bbar, then [Na] alpha or ln(alpha/abar)
-    const float *__restrict__ prow = r.pts32 + (size_t)tile * r.pts_rows * TILE_M + tid;
+    const float *prow = r.pts32 + (size_t)tile * r.pts_rows * TILE_M + tid;
     const int64_t p = (int64_t)tile * TILE_M + tid;   // the point whose weights and sums this thread owns
     const bool inb = p < r.P;
     const int TCr = r.simt_tc;
@@ -927,8 +927,8 @@ __global__ void __launch_bounds__(SIMT_THREADS) simt_kernel(const ReqDesc *__res
 #pragma unroll
                 for (int u = 0; u < SIMT_WU; ++u) {
                     if (i0 + u < N) {
-                        b[u] = __ldg(prow + j * TILE_M);
-                        a[u] = Na ? __ldg(pa) : 0.0f;
+                        b[u] = prow[j * TILE_M];
+                        a[u] = Na ? pa[0] : 0.0f;
                     } else {
                         b[u] = a[u] = 0.0f;
                     }
@@ -1127,7 +1127,7 @@ __device__ __forceinline__ void two_sum_acc(float &s, float &c, float x) {
 // When the launch's status word is set (a bounded wait ran out, so some
 // partials were never written), every logL of the launch is NaN.
 template <bool WARP>
-__global__ void __launch_bounds__(REDUCE_THREADS) reduce_kernel(const ReqDesc *__restrict__ reqs, int n_reqs) {
+__global__ void __launch_bounds__(REDUCE_THREADS) reduce_kernel(const ReqDesc *reqs, int n_reqs) {
     pdl_wait();
     const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t gid = WARP ? tid >> 5 : tid;
@@ -1143,7 +1143,7 @@ __global__ void __launch_bounds__(REDUCE_THREADS) reduce_kernel(const ReqDesc *_
     const unsigned char valid = r.pvalid[p];       // the statistics pass tested the point (point_valid)
     const double2 nm = r.pnorm ? r.pnorm[p] : make_double2(0.0, 0.0);
     float sh = 0.0f, sl = 0.0f;
-    const float2 *__restrict__ part = r.partials + (size_t)p * r.n_part;
+    const float2 *part = r.partials + (size_t)p * r.n_part;
     constexpr int UN = WARP ? 4 : 16, STEP = WARP ? 32 : 1;
     for (int g0 = lane; g0 < r.n_part; g0 += UN * STEP) {
         float2 v[UN];
@@ -1183,7 +1183,7 @@ __global__ void __launch_bounds__(REDUCE_THREADS) reduce_kernel(const ReqDesc *_
 
 // Validation helper: T_model[p,f,t] with the arithmetic of the SIMT forms.
 template <bool DIRECT>
-__global__ void model_eval_simt_kernel(const ReqDesc *__restrict__ req, double *__restrict__ out) {
+__global__ void model_eval_simt_kernel(const ReqDesc *req, double *__restrict__ out) {
     const ReqDesc &r = *req;
     const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t total = r.P * r.F * r.T;
@@ -1221,7 +1221,7 @@ __global__ void model_eval_simt_kernel(const ReqDesc *__restrict__ req, double *
     }
 }
 
-__global__ void resid_to_model_kernel(const ReqDesc *__restrict__ req, const float *__restrict__ resid,
+__global__ void resid_to_model_kernel(const ReqDesc *req, const float *__restrict__ resid,
                                       double *__restrict__ out) {
     const ReqDesc &r = *req;
     const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;

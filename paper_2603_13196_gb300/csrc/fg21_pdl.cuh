@@ -10,6 +10,13 @@
 // ordinary way.  No kernel triggers its dependents early: measured, the
 // dependents' blocks then sit on the SMs beside the running kernel and cost
 // more than the overlap gains.
+//
+// What the earlier kernels of the chain write (a call's only descriptor among
+// it) is read by plain loads, after the wait.  Neither __restrict__ on a kernel's
+// pointer to it nor __ldg may be used: both declare the memory unchanging while
+// the kernel runs, which it is not (the kernel may be resident before the one
+// that writes it has finished), and the compiler may then move a load whose
+// address it knows to before the wait.
 #pragma once
 #include <cuda_runtime.h>
 #include <utility>
