@@ -254,8 +254,13 @@ int fg21_loglike_batch(fg21_model *m, const double *params, int64_t P, double *l
 /* As fg21_loglike_batch with DEVICE buffers d_params [P][N+4] and d_logL [P],
  * enqueued asynchronously on `stream` (nothing is copied to or from the host;
  * the call returns before the kernels finish).  The model's workspace is
- * reused by the next call on the same model, which must be ordered after this
- * one (same stream, or synchronised).  The device-side invalid count and any
+ * reused by the next call on the same model; a call on another stream waits on
+ * the GPU for the one before it, so such calls never overlap (the buffers they
+ * share, d_logL say, remain the caller's to order).  A stream that is being
+ * captured is refused with FG21_E_CUDA before anything is allocated or enqueued,
+ * and the capture stays intact (also by fg21_loglike_batch, _multi, fg21_autotune
+ * and fg21_model_eval): use fg21_graph_create, or
+ * fg21_loglike_batch_device_noalloc.  The device-side invalid count and any
  * kernel failure are read by fg21_model_sync_status. */
 int fg21_loglike_batch_device(fg21_model *m, const double *d_params, int64_t P, double *d_logL,
                               int precision, void *stream);

@@ -94,12 +94,6 @@ int Workspace::ensure(size_t dev_need, size_t arena_need, size_t pinned_need, in
 // unless it was made on the same stream.  (Streams are told apart by their id,
 // which is never used twice, not by the handle.)
 int Workspace::order_after(cudaStream_t stream) {
-    // a call of this kind cannot be captured into a caller's graph: its workspace
-    // may be replaced by any later call
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    FG21_CUDA_TRY(cudaStreamIsCapturing(stream, &cap));
-    if (cap != cudaStreamCaptureStatusNone)
-        return set_error(FG21_E_CUDA, "the stream is being captured (fg21_graph_create captures an evaluation)");
     unsigned long long id = 0;
     FG21_CUDA_TRY(cudaStreamGetId(stream, &id));
     if (called && id != last_stream) FG21_CUDA_TRY(cudaStreamWaitEvent(stream, done, 0));
@@ -366,9 +360,22 @@ int launch_requests(Workspace &ws, const std::vector<ReqDesc> &reqs, const Prepa
     return FG21_OK;
 }
 
+// A call on a model's or the library's own workspace cannot become part of a
+// caller's graph: any later call may replace the workspace.  Asked before anything
+// is allocated, waited for or enqueued, so that the capture stays intact.
+int refuse_capture(cudaStream_t stream) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    FG21_CUDA_TRY(cudaStreamIsCapturing(stream, &cap));
+    if (cap != cudaStreamCaptureStatusNone)
+        return set_error(FG21_E_CUDA, "the stream is being captured (fg21_graph_create captures an evaluation)");
+    return FG21_OK;
+}
+
 int enqueue_requests(Workspace &ws, std::vector<ReqDesc> &reqs, int precision, cudaStream_t stream) {
+    int rc = refuse_capture(stream);
+    if (rc) return rc;
     Prepared pp;
-    int rc = prepare_requests(ws, reqs, precision, pp);
+    rc = prepare_requests(ws, reqs, precision, pp);
     if (rc || pp.n == 0) return rc;
     rc = ws.order_after(stream);
     if (rc) return rc;
@@ -506,6 +513,8 @@ static int run_host(fg21_model *m, const double *params, int64_t P, double *logL
                     cudaStream_t stream) {
     const size_t pbytes = sizeof(double) * (size_t)P * m->n_params(), lbytes = sizeof(double) * (size_t)P;
     const size_t need = align256(pbytes) + align256(lbytes) + 64;
+    int rc = refuse_capture(stream);
+    if (rc) return rc;
     if (m->io_cap < need) {
         if (m->ws.done) FG21_CUDA_TRY(cudaEventSynchronize(m->ws.done));
         if (m->host_graph) {
@@ -551,20 +560,20 @@ static int run_host(fg21_model *m, const double *params, int64_t P, double *logL
                 m->host_graph = nullptr;
             }
             fg21_graph *g = nullptr;
-            int rc = fg21_graph_create(m, io->d_params, P, io->d_logL, precision, &g);
+            rc = fg21_graph_create(m, io->d_params, P, io->d_logL, precision, &g);
             if (rc) return rc;
             m->host_graph = g;
             m->hg_P = P;
             m->hg_prec = precision;
             m->hg_cpg = cpg;
         }
-        int rc = fg21_graph_launch(m->host_graph, stream);
+        rc = fg21_graph_launch(m->host_graph, stream);
         if (rc) return rc;
         d_status = graph_status(m->host_graph);
     } else {
         // first calls of a size, and timed calls (fg21_model_timing, so that each
         // kernel is bracketed), launch directly
-        int rc = enqueue_requests(m->ws, reqs, precision, stream);
+        rc = enqueue_requests(m->ws, reqs, precision, stream);
         if (rc) return rc;
         d_status = m->ws.d_status;
     }
@@ -690,6 +699,8 @@ int fg21_autotune(fg21_model *m, const double *d_params, int64_t P, double *d_lo
     rc = device_guard(m);
     if (rc) return rc;
     cudaStream_t s = (cudaStream_t)stream;
+    rc = refuse_capture(s);
+    if (rc) return rc;
     // candidates: every distinct channels-per-group value that splits the
     // channels into 1..32 groups, plus the planner's model choice
     std::vector<int> cand;
@@ -864,6 +875,8 @@ int fg21_model_eval(fg21_model *m, const double *params, int64_t P, double *T_mo
     rc = device_guard(m);
     if (rc) return rc;
     cudaStream_t s = (cudaStream_t)stream;
+    rc = refuse_capture(s);
+    if (rc) return rc;
     const size_t pbytes = sizeof(double) * (size_t)P * m->n_params();
     const size_t obytes = sizeof(double) * (size_t)P * m->F * m->T;
     double *d_params = nullptr, *d_out = nullptr, *d_logL = nullptr;
@@ -921,6 +934,8 @@ int fg21_loglike_multi(fg21_model *const *models, const double *const *params, c
     static size_t io_cap = 0;
     std::lock_guard<std::mutex> lk(mu);
     cudaStream_t s = (cudaStream_t)stream;
+    int rc = refuse_capture(s);
+    if (rc) return rc;
     std::vector<size_t> poff(n_models), loff(n_models);
     size_t total = 0;
     for (int k = 0; k < n_models; ++k) {
@@ -956,7 +971,7 @@ int fg21_loglike_multi(fg21_model *const *models, const double *const *params, c
     if (reqs.empty()) return FG21_OK;
     FG21_CUDA_TRY(cudaMemcpyAsync(d_io, h_io, loff[n_models - 1] + align256(sizeof(double) * P[n_models - 1]),
                                   cudaMemcpyHostToDevice, s));
-    int rc = enqueue_requests(ws, reqs, precision, s);
+    rc = enqueue_requests(ws, reqs, precision, s);
     if (rc) return rc;
     FG21_CUDA_TRY(cudaMemcpyAsync(h_io, d_io, total - 64, cudaMemcpyDeviceToHost, s));
     unsigned st[8];

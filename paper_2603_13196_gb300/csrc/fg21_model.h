@@ -49,6 +49,8 @@ inline size_t status_bytes(int) { return 32; }
 // main and reduce kernels on `stream`.  The status word and invalid counter
 // are cleared first.  Returns FG21_OK or an error code.
 int enqueue_requests(Workspace &ws, std::vector<ReqDesc> &reqs, int precision, cudaStream_t stream);
+// FG21_E_CUDA if `stream` is being captured.
+int refuse_capture(cudaStream_t stream);
 
 // The two halves of enqueue_requests: plan, size the workspace, carve and fill
 // the descriptors (staged in ws.pinned) ...
