@@ -158,6 +158,11 @@ int fg21_device_count(void);
  * its data vector is zero until fg21_model_set_data.  labels_out [npix] and
  * edges_out [N+1] are optional (may be NULL).  The library copies what it
  * needs; inputs may be freed on return.
+ * While it runs, the build holds device memory besides the model's: tables of
+ * (2 F + T) npix doubles and A, and, if a quarter of the free memory has room for
+ * it, the beam (F T npix doubles: 11.8 GB at 49152 pixels, 301 channels, 100 bins).
+ * The beam is given back when another of the build's allocations needs the room;
+ * without it the results are the same, bit for bit, and the build takes longer.
  * Errors: FG21_E_ARG (NULL input, N < 1 or N > npix or N > FG21_MAX_REGIONS,
  * F, T, npix <= 0, nu <= 0, beam_p < 0, |v| or |z| not within 1e-6 of 1,
  * unknown scheme/weighting), FG21_E_NOMEM, FG21_E_CUDA. */
@@ -196,6 +201,17 @@ int fg21_build_regions_ab(const fg21_sky *sky, const fg21_obs *obs, const fg21_p
 int fg21_build_regions_ab_host(const fg21_sky *sky, const fg21_obs *obs, const fg21_partition_opts *beta_opt,
                                const fg21_amplitude_opts *alpha_opt, int32_t *beta_labels, double *beta_edges,
                                int32_t *alpha_labels, double *alpha_edges, double *K_out, double *B_out);
+
+/* The paper has no counterpart to this call: it checks region building where
+ * device memory is short.  As fg21_build_regions (alpha_opt NULL) or
+ * fg21_build_regions_ab, with at most limit_bytes of device memory for the build
+ * (0: as much as there is; the model itself is not counted): FG21_E_NOMEM when the
+ * build does not fit without the beam either.  *beam_use (may be NULL): 0 the beam
+ * had no room, 1 it was kept, 2 it was given back.  labels, edges, A and B do not
+ * depend on it. */
+int fg21_selftest_build_regions(const fg21_sky *sky, const fg21_obs *obs, const fg21_partition_opts *beta_opt,
+                                const fg21_amplitude_opts *alpha_opt, size_t limit_bytes, fg21_model **out,
+                                int32_t *beta_labels, double *beta_edges, int32_t *beam_use);
 
 /* Parameter layout of a model: spectral-index regions, amplitude parameters
  * (0 for models of fg21_build_regions) and values per parameter row

@@ -21,8 +21,8 @@
 // What bounds it is the FP64 exponential of D (this part's FP64 rate is 1/64 of
 // FP32's), needed by every pass: pass 1 keeps D [F][T][Npix] in device memory
 // where a quarter of what is free holds it (0.3 GB at 12288 pixels, 151 channels, 20
-// bins; 11.8 GB at 49152, 301, 100) and the others read it; without the room they
-// evaluate it again.  The tables of one build serve both its halves.
+// bins; 11.8 GB at 49152, 301, 100) and the others read it; without the room, or
+// when another allocation of the build needs it, they evaluate it again.  The tables of one build serve both its halves.
 // 12288 pixels, 9 regions, 151 channels, 20 bins: 4.06 ms a build from 8.00 (four
 // evaluations of D, and the tables made twice).
 #include <cuda_runtime.h>
@@ -179,36 +179,75 @@ int fail(cudaError_t e, const char *what) {
 }  // namespace
 
 // Device copies of the inputs, the geometry tables and the beam of one build,
-// freed on destruction.
+// freed on destruction.  What the build can do without, the beam, and, for its
+// second half, the tables of the importance weights, is given back when another
+// allocation fails for lack of memory.
 struct DeviceBuild {
     const fg21_sky *s;
     const fg21_obs *o;
+    size_t limit;            // most device bytes the build may hold (0: as many as there are)
+    size_t held = 0;
     DevObs g{};
     double *t230 = nullptr, *beta = nullptr, *lognu = nullptr, *tsky = nullptr, *beam = nullptr;
-    double *inv_den = nullptr, *bsum = nullptr;
+    double *inv_den = nullptr, *bsum = nullptr, *pw = nullptr, *w = nullptr;
     bool ready = false, summed = false;      // tables made; bsum (and beam) written
-    std::vector<void *> own;
+    bool weighted = false;                   // no importance weights are needed any more
+    int beam_use = 0;                        // 0: the beam had no room, 1: kept, 2: given back
+    std::vector<std::pair<void *, size_t>> own;
     ~DeviceBuild() {
-        for (void *p : own) cudaFree(p);
+        for (auto &p : own) cudaFree(p.first);
+    }
+    template <typename T>
+    cudaError_t try_alloc(T **p, size_t n) {
+        *p = nullptr;
+        const size_t bytes = sizeof(T) * n;
+        if (limit && held + bytes > limit) return cudaErrorMemoryAllocation;
+        cudaError_t e = cudaMalloc((void **)p, bytes);
+        if (e == cudaErrorMemoryAllocation) cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        own.emplace_back(*p, bytes);
+        held += bytes;
+        return e;
+    }
+    // Frees what the rest of the build can do without (cudaFree waits for the
+    // kernels that use it); true if there was any.
+    bool shed() {
+        const size_t before = own.size();
+        if (beam) {
+            drop(beam);
+            beam_use = 2;
+        }
+        g.D = nullptr;
+        if (weighted) {
+            drop(pw);
+            drop(w);
+            drop(tsky);
+            g.tskyT = nullptr;
+        }
+        return own.size() < before;
+    }
+    void drop(double *&p) {
+        for (size_t k = 0; p && k < own.size(); ++k)
+            if (own[k].first == p) {
+                cudaFree(p);
+                held -= own[k].second;
+                own.erase(own.begin() + k);
+                p = nullptr;
+            }
     }
     template <typename T>
     cudaError_t alloc(T **p, size_t n) {
-        cudaError_t e = cudaMalloc((void **)p, sizeof(T) * n);
-        if (e == cudaSuccess) own.push_back(*p);
+        cudaError_t e = try_alloc(p, n);
+        if (e == cudaErrorMemoryAllocation && shed()) e = try_alloc(p, n);
         return e;
+    }
+    cudaError_t upload(double **dst, const double *src, size_t n) {
+        const cudaError_t e = alloc(dst, n);
+        return e != cudaSuccess ? e : cudaMemcpy(*dst, src, sizeof(double) * n, cudaMemcpyHostToDevice);
     }
     cudaError_t prepare(bool need_tsky);
     cudaError_t pass1(int weighting);
 };
-
-namespace {
-cudaError_t upload(std::vector<void *> &own, double **dst, const double *src, size_t n) {
-    cudaError_t e = cudaMalloc((void **)dst, sizeof(double) * n);
-    if (e != cudaSuccess) return e;
-    own.push_back(*dst);
-    return cudaMemcpy(*dst, src, sizeof(double) * n, cudaMemcpyHostToDevice);
-}
-}  // namespace
 
 // inputs, ln c per (t, q) and (when needed) T_sky per (f, q)
 cudaError_t DeviceBuild::prepare(bool need_tsky) {
@@ -219,12 +258,12 @@ cudaError_t DeviceBuild::prepare(bool need_tsky) {
         std::vector<double> ln(F);
         for (int f = 0; f < F; ++f) ln[f] = std::log(o->nu[f] / o->nu0);
         double *dirs = nullptr, *zen = nullptr, *beam_p = nullptr, *logcT = nullptr;
-        e = upload(own, &dirs, s->dirs, 3 * (size_t)npix);
-        if (e == cudaSuccess) e = upload(own, &t230, s->t230, npix);
-        if (e == cudaSuccess) e = upload(own, &beta, s->beta, npix);
-        if (e == cudaSuccess) e = upload(own, &lognu, ln.data(), F);
-        if (e == cudaSuccess) e = upload(own, &beam_p, o->beam_p, F);
-        if (e == cudaSuccess) e = upload(own, &zen, o->zenith, 3 * (size_t)T);
+        e = upload(&dirs, s->dirs, 3 * (size_t)npix);
+        if (e == cudaSuccess) e = upload(&t230, s->t230, npix);
+        if (e == cudaSuccess) e = upload(&beta, s->beta, npix);
+        if (e == cudaSuccess) e = upload(&lognu, ln.data(), F);
+        if (e == cudaSuccess) e = upload(&beam_p, o->beam_p, F);
+        if (e == cudaSuccess) e = upload(&zen, o->zenith, 3 * (size_t)T);
         if (e == cudaSuccess) e = alloc(&logcT, (size_t)npix * T);
         if (e == cudaSuccess) e = alloc(&inv_den, (size_t)F * T);
         if (e == cudaSuccess) e = alloc(&bsum, (size_t)F * T);
@@ -241,11 +280,13 @@ cudaError_t DeviceBuild::prepare(bool need_tsky) {
         g.t_cmb = o->t_cmb;
         // room for the beam: at most a quarter of the free memory, and no error without it
         const size_t need = sizeof(double) * (size_t)npix * F * T;
-        size_t free_bytes = 0, total = 0;
-        if (cudaMemGetInfo(&free_bytes, &total) == cudaSuccess && need <= free_bytes / 4 &&
-            alloc(&beam, (size_t)npix * F * T) != cudaSuccess)
-            beam = nullptr;
-        cudaGetLastError();
+        size_t room = 0, total = 0;
+        if (cudaMemGetInfo(&room, &total) != cudaSuccess) {
+            cudaGetLastError();
+            room = 0;
+        }
+        if (limit) room = std::min(room, limit);
+        if (need <= room / 4 && try_alloc(&beam, (size_t)npix * F * T) == cudaSuccess) beam_use = 1;
         ready = true;
     }
     if (need_tsky && !tsky) {
@@ -268,13 +309,15 @@ cudaError_t DeviceBuild::pass1(int weighting) {
     return e;
 }
 
-DeviceBuild *device_build_begin(const fg21_sky *s, const fg21_obs *o) {
+DeviceBuild *device_build_begin(const fg21_sky *s, const fg21_obs *o, size_t limit) {
     DeviceBuild *b = new DeviceBuild;
     b->s = s;
     b->o = o;
+    b->limit = limit;
     return b;
 }
 void device_build_end(DeviceBuild *b) { delete b; }
+int device_build_beam(const DeviceBuild *b) { return b->beam_use; }
 
 int device_importance(DeviceBuild *b, int weighting, std::vector<double> &w) {
     const bool need_tsky = weighting == FG21_WEIGHT_BEAM || weighting == FG21_WEIGHT_SKY;
@@ -282,22 +325,23 @@ int device_importance(DeviceBuild *b, int weighting, std::vector<double> &w) {
     if (e != cudaSuccess) return fail(e, "region building (inputs)");
     const int64_t npix = b->g.npix;
     const int F = b->g.F, T = b->g.T, th = BUILD_THREADS;
-    double *pw = nullptr, *dw = nullptr;
-    e = b->alloc(&pw, (size_t)F * npix);
-    if (e == cudaSuccess) e = b->alloc(&dw, (size_t)npix);
+    // (kept for the build's other weighting, if it has one)
+    if (!b->pw) e = b->alloc(&b->pw, (size_t)F * npix);
+    if (e == cudaSuccess && !b->w) e = b->alloc(&b->w, (size_t)npix);
     if (e != cudaSuccess) return fail(e, "region building (importance)");
     if ((e = b->pass1(weighting)) != cudaSuccess) return fail(e, "den_kernel");
-    pw_kernel<<<dim3((unsigned)((npix + th - 1) / th), (unsigned)F), th>>>(b->g, weighting, b->inv_den, pw);
-    w_kernel<<<(unsigned)((npix + th - 1) / th), th>>>(pw, npix, F, 1.0 / ((double)F * (double)T), dw);
+    pw_kernel<<<dim3((unsigned)((npix + th - 1) / th), (unsigned)F), th>>>(b->g, weighting, b->inv_den, b->pw);
+    w_kernel<<<(unsigned)((npix + th - 1) / th), th>>>(b->pw, npix, F, 1.0 / ((double)F * (double)T), b->w);
     if ((e = cudaGetLastError()) != cudaSuccess) return fail(e, "w_kernel");
     w.resize(npix);
-    if ((e = cudaMemcpy(w.data(), dw, sizeof(double) * npix, cudaMemcpyDeviceToHost)) != cudaSuccess)
+    if ((e = cudaMemcpy(w.data(), b->w, sizeof(double) * npix, cudaMemcpyDeviceToHost)) != cudaSuccess)
         return fail(e, "region building (w)");
     return FG21_OK;
 }
 
 int device_precompute(DeviceBuild *b, const std::vector<int32_t> &lab, int N, std::vector<double> &A,
                       std::vector<double> &B) {
+    b->weighted = true;
     cudaError_t e = b->prepare(false);
     if (e != cudaSuccess) return fail(e, "region building (inputs)");
     const int64_t npix = b->g.npix;

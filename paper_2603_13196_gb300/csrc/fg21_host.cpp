@@ -356,6 +356,7 @@ struct Built {
     std::vector<int32_t> lab, lab_a;
     int Nb = 0, Na = 0;          // Na = 0: no amplitude regions
     int n_empty = 0;             // components without a pixel
+    int beam_use = 0;            // device builds: device_build_beam
 };
 
 int check_opts(const fg21_sky *sky, int N, int scheme, int weighting, const char *what) {
@@ -382,9 +383,10 @@ void partition_field(int64_t npix, const double *field, const std::vector<double
 // Spectral-index regions (opt), optionally amplitude regions (aopt), and the
 // response functions of their intersections: component i * Nb + j.  With
 // `device` the O(Npix F T) sums (importance weights, response functions) run
-// on the current GPU (fg21_build.cu); the partition is the same host code.
+// on the current GPU (fg21_build.cu), in at most device_limit bytes (0: no limit);
+// the partition is the same host code.
 int build_host(const fg21_sky *sky, const fg21_obs *obs, const fg21_partition_opts *opt,
-               const fg21_amplitude_opts *aopt, Built &out, bool device) {
+               const fg21_amplitude_opts *aopt, Built &out, bool device, size_t device_limit = 0) {
     if (!opt) return set_error(FG21_E_ARG, "NULL opt");
     int rc = check_inputs(sky, obs);
     if (rc) return rc;
@@ -406,8 +408,7 @@ int build_host(const fg21_sky *sky, const fg21_obs *obs, const fg21_partition_op
     const int N = std::max(Na, 1) * Nb;
     try {
         Geometry g;
-        std::unique_ptr<DeviceBuild, void (*)(DeviceBuild *)> dev(device ? device_build_begin(sky, obs) : nullptr,
-                                                                  device_build_end);
+        std::unique_ptr<DeviceBuild, void (*)(DeviceBuild *)> dev(device ? device_build_begin(sky, obs, device_limit) : nullptr, device_build_end);
         if (!device) build_geometry(sky, obs, g);
         auto weights = [&](int weighting, std::vector<double> &w) -> int {
             if (device) return device_importance(dev.get(), weighting, w);
@@ -427,6 +428,7 @@ int build_host(const fg21_sky *sky, const fg21_obs *obs, const fg21_partition_op
         }
         if (device) {
             if ((rc = device_precompute(dev.get(), comp, N, out.A, out.B))) return rc;
+            out.beam_use = device_build_beam(dev.get());
         } else {
             precompute(sky, obs, g, comp, N, out.A, out.B);
         }
@@ -534,6 +536,21 @@ int fg21_build_regions_ab(const fg21_sky *sky, const fg21_obs *obs, const fg21_p
     if (beta_edges) std::memcpy(beta_edges, b.edges.data(), sizeof(double) * b.edges.size());
     if (alpha_labels) std::memcpy(alpha_labels, b.lab_a.data(), sizeof(int32_t) * b.lab_a.size());
     if (alpha_edges) std::memcpy(alpha_edges, b.edges_a.data(), sizeof(double) * b.edges_a.size());
+    return make_model(sky, obs, b, out);
+}
+
+int fg21_selftest_build_regions(const fg21_sky *sky, const fg21_obs *obs, const fg21_partition_opts *beta_opt,
+                                const fg21_amplitude_opts *alpha_opt, size_t limit_bytes, fg21_model **out,
+                                int32_t *beta_labels, double *beta_edges, int32_t *beam_use) {
+    clear_error();
+    if (!out) return set_error(FG21_E_ARG, "NULL out");
+    *out = nullptr;
+    Built b;
+    int rc = build_host(sky, obs, beta_opt, alpha_opt, b, true, limit_bytes);
+    if (rc) return rc;
+    if (beta_labels) std::memcpy(beta_labels, b.lab.data(), sizeof(int32_t) * b.lab.size());
+    if (beta_edges) std::memcpy(beta_edges, b.edges.data(), sizeof(double) * b.edges.size());
+    if (beam_use) *beam_use = b.beam_use;
     return make_model(sky, obs, b, out);
 }
 

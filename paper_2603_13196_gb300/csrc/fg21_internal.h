@@ -201,10 +201,12 @@ int tc_map_init();  // resolves cuTensorMapEncodeTiled; FG21_OK or error
 // build shared by its halves: the importance weights w[npix] of `weighting`
 // (Sec. 4.2), and the response functions A[N][F][T] of the components `lab`
 // (Sec. 2.2 eq. chromatic_function) with B[F][T].  Same FP64 arithmetic as the
-// host code, other summation order.  FG21_OK or an error code (message set).
+// host code, other summation order.  `limit`: most device bytes a build may hold
+// (0: as many as there are).  FG21_OK or an error code (message set).
 struct DeviceBuild;
-DeviceBuild *device_build_begin(const fg21_sky *s, const fg21_obs *o);
+DeviceBuild *device_build_begin(const fg21_sky *s, const fg21_obs *o, size_t limit);
 void device_build_end(DeviceBuild *b);
+int device_build_beam(const DeviceBuild *b);   // 0: the beam had no room, 1: kept, 2: given back
 int device_importance(DeviceBuild *b, int weighting, std::vector<double> &w);
 int device_precompute(DeviceBuild *b, const std::vector<int32_t> &lab, int N, std::vector<double> &A,
                       std::vector<double> &B);

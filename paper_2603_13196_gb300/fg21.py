@@ -91,6 +91,7 @@ _SIGS = {
     "fg21_model_sync_status": (C.c_int, [_P, _P, _P]),
     "fg21_selftest_bounded_wait": (C.c_int, [_P, _P, _P]),
     "fg21_selftest_mma_rounding": (C.c_int, [_P, _P, _P, _P, _P]),
+    "fg21_selftest_build_regions": (C.c_int, [_P, _P, _P, _P, C.c_size_t, _P, _P, _P, _P]),
     "fg21_autotune": (C.c_int, [_P, _P, C.c_int64, _P, C.c_int, _P, _P, _P]),
     "fg21_model_eval": (C.c_int, [_P, _P, C.c_int64, _P, C.c_int, _P]),
     "fg21_model_timing": (C.c_int, [_P, C.c_int]),
@@ -284,6 +285,23 @@ def fg21_build_regions_ab_host(sky, obs, n_beta: int, scheme, weighting, n_alpha
                                             _ptr(edges), _ptr(lab_a), _ptr(edges_a), _ptr(K), _ptr(B)),
            "fg21_build_regions_ab_host")
     return lab, edges, lab_a, edges_a, K, B
+
+
+def fg21_selftest_build_regions(sky, obs, n_beta: int, limit_bytes: int = 0, weighting="beam", n_alpha: int = 0,
+                                field=None, weighting_a="beam"):
+    """-> (Model, beam use) of a device build in at most limit_bytes (0: no limit);
+    recursive regions, and with n_alpha amplitude regions of `field`."""
+    k = _Keep(sky, obs)
+    opt = fg21_partition_opts(n_beta, SCHEMES["recursive"], WEIGHTINGS[weighting])
+    aopt, keep = _amp_opts(n_alpha, "recursive", weighting_a, field) if n_alpha else (None, None)
+    out, use = C.c_void_p(), C.c_int32(-1)
+    lab = np.empty(k.sky.npix, dtype=np.int32)
+    edges = np.empty(n_beta + 1)
+    _check(lib().fg21_selftest_build_regions(C.byref(k.sky), C.byref(k.obs), C.byref(opt),
+                                             C.byref(aopt) if aopt is not None else None, int(limit_bytes),
+                                             C.byref(out), _ptr(lab), _ptr(edges), C.byref(use)),
+           "fg21_selftest_build_regions")
+    return Model(out.value, max(n_alpha, 1) * n_beta, k.obs.F, k.obs.T, lab, edges, Nb=n_beta, Na=n_alpha), use.value
 
 
 def fg21_model_shape(m: Model) -> dict:
