@@ -352,11 +352,12 @@ int fg21_selftest_mma_rounding(const uint16_t *a, const uint16_t *b, const float
 /* Measured choice of the work split of requests of P points of model m at
  * `precision` (the number of channels per work item of the batched
  * evaluation of eq. likelihood over eq. fast_forward_model): runs one
- * evaluation per candidate split (every distinct channels-per-item value that
- * cuts the F channels into 1..32 groups) five times on the caller's DEVICE
- * buffers d_params [P][N+4] / d_logL [P] (d_logL is overwritten with valid
- * results), times the last four with CUDA events on `stream`, keeps the split
- * with the smallest median in the model and returns it (and its time in ms).
+ * evaluation per candidate split (the planner's own, and every distinct
+ * channels-per-item value that cuts the F channels into 1..32 groups) five
+ * times on the caller's DEVICE buffers d_params [P][N+4] / d_logL [P] (d_logL is
+ * overwritten with valid results), times the last four with CUDA events on
+ * `stream`, keeps the split with the smallest median in the model and returns
+ * it (and its time in ms).
  * Every later plan of model m at `precision` for the same number of 128-point
  * tiles (alone, batched, served or captured in a graph) uses it, so a
  * request's results still depend only on its own model and size.  Blocks

@@ -701,9 +701,16 @@ int fg21_autotune(fg21_model *m, const double *d_params, int64_t P, double *d_lo
     cudaStream_t s = (cudaStream_t)stream;
     rc = refuse_capture(s);
     if (rc) return rc;
-    // candidates: every distinct channels-per-group value that splits the
-    // channels into 1..32 groups, plus the planner's model choice
+    // candidates: the planner's own split first, then every distinct
+    // channels-per-group value that splits the channels into 1..32 groups (the
+    // planner has no such limit: 128 points, 151 channels, one channel an item)
     std::vector<int> cand;
+    {
+        ReqDesc r = model_request(m, d_params, P, d_logL, precision);
+        r.cpg_hint = 0;
+        plan_request(r, precision, num_sms_of(m->device), (P + TILE_M - 1) / TILE_M);
+        cand.push_back(r.ch_per_group);
+    }
     for (int G = 1; G <= std::min(m->F, 32); ++G) {
         const int cpg = (m->F + G - 1) / G;
         if (std::find(cand.begin(), cand.end(), cpg) == cand.end()) cand.push_back(cpg);
