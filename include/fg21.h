@@ -288,8 +288,8 @@ int fg21_loglike_batch_device(fg21_model *m, const double *d_params, int64_t P, 
  * allocate GPU memory while they evaluate the likelihood: a host application
  * that gives the library a fixed device-memory budget at start-up and forbids
  * growth afterwards, or a runtime that owns the GPU's memory pool and refuses
- * allocations from plug-ins once it is running.  Same arguments and results as
- * fg21_loglike_batch_device, for the tensor-core precisions (FG21_PREC_FP16X3,
+ * allocations from plug-ins once it is running.  Same arguments and results (bit
+ * for bit) as fg21_loglike_batch_device, for the tensor-core precisions (FG21_PREC_FP16X3,
  * FG21_PREC_BF16X3), but it calls no cudaMalloc / cudaFree and allocates
  * nothing: all per-call scratch, the request descriptor included, comes from
  * one static device array of FG21_NOALLOC_SCRATCH_BYTES (32 MiB) that every GPU

@@ -46,7 +46,8 @@ __host__ __device__ inline size_t fused_doubles(int P, int Rp) {
     return ((size_t)P * Rp + (P + 7) / 8 + 1) / 2 * 2;
 }
 __device__ __forceinline__ double *fused_slab(double *base, int P, int Rp) { return base + fused_doubles(P, Rp); }
-constexpr int REDUCE_THREADS = 64;
+constexpr int REDUCE_THREADS = 64;           // (divides a tile: a grid over whole tiles has no point beyond them)
+static_assert(TILE_M % REDUCE_THREADS == 0, "see the allocation-free call's parts");
 constexpr int REDUCE_SERIAL_MAX = 32;       // longest partial row summed by one thread
 
 // A point is valid when all its parameters are finite, sigma_n > 0,
