@@ -38,12 +38,8 @@ void graph_free(fg21_graph *g) {
 
 }  // namespace
 
-unsigned *fg21::graph_status(fg21_graph *g) { return g->ws.d_status; }
-
-extern "C" {
-
-int fg21_graph_create_multi(fg21_model *const *models, const double *const *d_params, const int64_t *P,
-                            double *const *d_logL, int n_models, int precision, fg21_graph **out) {
+static int graph_create(fg21_model *const *models, const double *const *d_params, const int64_t *P,
+                        double *const *d_logL, int n_models, int precision, unsigned *d_status, fg21_graph **out) {
     if (!out) return set_error(FG21_E_ARG, "NULL output");
     *out = nullptr;
     if (n_models <= 0 || !models || !d_params || !P || !d_logL) return set_error(FG21_E_ARG, "bad graph arguments");
@@ -52,6 +48,7 @@ int fg21_graph_create_multi(fg21_model *const *models, const double *const *d_pa
     FG21_CUDA_TRY(cudaGetDevice(&dev));
     fg21_graph *g = new fg21_graph;
     g->device = dev;
+    if (d_status) g->ws.borrow_status(d_status);
     for (int k = 0; k < n_models; ++k) {
         fg21_model *m = models[k];
         if (!m || P[k] < 0 || (P[k] > 0 && (!d_params[k] || !d_logL[k]))) {
@@ -102,6 +99,18 @@ int fg21_graph_create_multi(fg21_model *const *models, const double *const *d_pa
     }
     *out = g;
     return FG21_OK;
+}
+
+int fg21::graph_create_on(fg21_model *m, const double *d_params, int64_t P, double *d_logL, int precision,
+                          unsigned *d_status, fg21_graph **out) {
+    return graph_create(&m, &d_params, &P, &d_logL, 1, precision, d_status, out);
+}
+
+extern "C" {
+
+int fg21_graph_create_multi(fg21_model *const *models, const double *const *d_params, const int64_t *P,
+                            double *const *d_logL, int n_models, int precision, fg21_graph **out) {
+    return graph_create(models, d_params, P, d_logL, n_models, precision, nullptr, out);
 }
 
 int fg21_graph_create(fg21_model *m, const double *d_params, int64_t P, double *d_logL, int precision,

@@ -25,6 +25,12 @@ struct Workspace {
     int reqs_cap = 0;
     unsigned *d_status = nullptr;   // bytes 0..3 status word, 16..23 invalid counter
     unsigned long long *d_invalid = nullptr;
+    bool own_status = true;         // false: the status block is the caller's (borrow_status)
+    void borrow_status(unsigned *block) {
+        d_status = block;
+        d_invalid = (unsigned long long *)((char *)block + 16);
+        own_status = false;
+    }
     cudaEvent_t done = nullptr;     // recorded after the last launch of a call
     bool called = false;            // ... which there has been
     unsigned long long last_stream = 0;   // id of that call's stream
@@ -105,6 +111,8 @@ int model_upload(fg21_model *m);
 // A request descriptor of model m for `precision` (carrying the autotuned work
 // split for its size, if any).
 ReqDesc model_request(fg21_model *m, const double *d_params, int64_t P, double *d_logL, int precision);
-// The device status word (and invalid count) of a graph's workspace.
-unsigned *graph_status(fg21_graph *g);
+// A graph of one model's evaluation whose status block (status_bytes) is the
+// caller's; it must outlive the graph.
+int graph_create_on(fg21_model *m, const double *d_params, int64_t P, double *d_logL, int precision,
+                    unsigned *d_status, fg21_graph **out);
 }  // namespace fg21
