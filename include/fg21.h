@@ -395,8 +395,8 @@ int fg21_loglike_multi(fg21_model *const *models, const double *const *params, c
  * Sec. 3).  fg21_graph_create_multi plans the batch of n_models requests
  * (model k, P[k] points, DEVICE buffers d_params[k] [P[k]][N_k+4] and
  * d_logL[k] [P[k]] on the current device), sizes a workspace owned by the
- * graph, uploads the request descriptors and captures one evaluation (status
- * clear, prep, tensor-core or SIMT kernel, reduction) into a CUDA graph.
+ * graph, uploads the request descriptors and captures one evaluation (prep,
+ * tensor-core or SIMT kernel, reduction) into a CUDA graph.
  * fg21_graph_launch replays it on `stream`; each replay reads the parameter
  * buffers as they are when it runs and writes the logL buffers, with the same
  * arithmetic (and the same results, bit for bit) as fg21_loglike_multi /

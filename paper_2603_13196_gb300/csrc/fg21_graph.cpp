@@ -2,9 +2,9 @@
 // capture one likelihood evaluation of a fixed set of requests (models, point
 // counts, device parameter and output buffers) into a CUDA graph once, and
 // fg21_graph_launch replays it.  The plan, workspace and request descriptors
-// are made and uploaded at creation; a replay is the status clear, the prep,
-// tensor-core (or SIMT) and reduction kernels, and reads whatever the
-// parameter buffers hold when it runs.  This is the batched evaluation of
+// are made and uploaded at creation; a replay is the prep (which clears the
+// status block), tensor-core (or SIMT) and reduction kernels, and reads whatever
+// the parameter buffers hold when it runs.  This is the batched evaluation of
 // eq. likelihood (Sec. 2.3.1) over eq. fast_forward_model (Sec. 2.2) for the
 // points a nested sampler proposes (Sec. 3), with the per-call host work and
 // launch latency taken out of the loop.

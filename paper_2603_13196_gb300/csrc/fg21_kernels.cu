@@ -41,7 +41,9 @@ constexpr int FUSED_POINTS = 256, FUSED_VALUES = 4096;
 __host__ __device__ inline bool request_fused(const ReqDesc &r) {
     return r.coef2 && r.P <= FUSED_POINTS && r.P * (r.NPF + 4) <= FUSED_VALUES;
 }
-// Start of a block's slab after the staged rows and validity bytes (16-byte aligned).
+// Doubles of the staged rows and validity bytes, which a block's slab follows: an
+// even number, so the slab is aligned as the rows are, to 8 bytes (what comes before
+// them, prep_head_doubles, is an odd number).
 __host__ __device__ inline size_t fused_doubles(int P, int Rp) {
     return ((size_t)P * Rp + (P + 7) / 8 + 1) / 2 * 2;
 }

@@ -180,8 +180,12 @@ static int choose_channels_per_group(int64_t total_tiles, int F, int slots, int 
 // two items at once: a CTA with m of the items takes about m / 2 rounds of two
 // and, for an odd m, one alone, which is 1.26 times as fast a stage as a pair
 // (0.54 against 0.68 us at 24 regions, 100 bins); an item costs about two stages
-// besides its own.  A stage is a channel's t-chunk.  Measured against counting
-// waves of single items (16384 points, 301 channels: the same split):
+// besides its own.  A stage is a channel's t-chunk.  Both numbers were fitted to
+// the times of 25 splits at 7 sizes.  Over 12 sizes of 1 to 32 tiles, 51 to 301
+// channels, 3 to 45 regions and 1 to 100 bins the split taken is the fastest of 13 to
+// within 0.1 us a replay, but for 128 points, 24 regions, 301 channels, 100 bins
+// (1 channel an item 26.7 us, 2 to 6 24.6) and 400 points, 3 regions, one bin (22.6,
+// 21.4 with 3).  Measured against counting waves of single items (16384 points, 301 channels: the same split):
 // 3001 points, 211 channels, two chunks 71 us a call from 78; 8192 points, 301
 // channels, amplitude regions 91 from 97; 4096 points, 151 channels 29.9 from 31.
 static int choose_channels_tc(int64_t tiles, int F, int n_tchunks, int num_sms) {
@@ -227,7 +231,7 @@ void plan_request(ReqDesc &r, int precision, int num_sms, int64_t total_tiles) {
     }
     r.G = (r.F + cpg - 1) / cpg;
     r.ch_per_group = (r.F + r.G - 1) / r.G;
-    r.n_part = tc ? 2 * r.G : r.G;      // the tensor path splits each point's t-columns over two warps
+    r.n_part = tc ? 2 * r.G : r.G;      // the tensor path sums each half of a point's t-columns by itself
     r.chi2_scale = tc ? 1.0 + (2.0 / 3.0) * std::ldexp(1.0, -23) : 1.0;
     r.tile_rows = (int64_t)r.Kp * r.Tc_pad / 32;   // 2 splits x Kp x Tc_pad x 2 bytes / 128
 }

@@ -45,7 +45,7 @@
 // latter also telling the producers that the slot is free.
 //
 // What bounds it: instruction issue and latency in the sixteen arithmetic warps
-// (FMA pipe about 58 % busy at 24 regions, 100 bins), so the stages are written
+// (FMA pipe about 54 % busy at 24 regions, 100 bins), so the stages are written
 // to spend few instructions besides the arithmetic and to depend on nothing
 // slow:
 //  - every role runs its loops warp-uniformly, and the elected lane issues MMAs,
@@ -812,8 +812,8 @@ __device__ __forceinline__ void issue_mmas(uint32_t d_tmem, uint32_t w_hi, uint3
                                            uint32_t b_lbo, uint32_t b_split, uint32_t idesc, uint32_t el) {
     // one descriptor for the stage's tile; each MMA adds its offset (16-byte
     // units) to the start-address field, which shared-memory addresses below
-    // 256 KB never carry out of (the issuing thread is busy about half the
-    // kernel's time in this sequence: building every descriptor afresh cost 3%)
+    // 256 KB never carry out of (building every descriptor afresh cost 3 % while one
+    // lane issued from a branch of its own; the issuers now wait 60-70 % of the time)
     const uint64_t d0 = smem_desc(b_addr, b_lbo, 128);
     const uint32_t step = (2 * b_lbo) >> 4, split = b_split >> 4;
 #pragma unroll
