@@ -348,9 +348,10 @@ __device__ __forceinline__ void begin_call(const ReqDesc &r, ReqDesc *store) {
 static_assert(sizeof(ReqDesc) % 8 == 0 && sizeof(ReqDesc) <= 2048, "the descriptor travels as a kernel argument");
 
 // ONE: the launch's only request, passed by value (stored at `store` unless
-// null); otherwise reqs[blockIdx.y].
+// null); otherwise reqs[blockIdx.y].  (reqs is read for several requests only,
+// whose descriptors were there before the call's first kernel: hence __restrict__.)
 template <bool ONE>
-__global__ void __launch_bounds__(STAT_BLOCK) prep_stats_kernel(const ReqDesc *reqs, int staged,
+__global__ void __launch_bounds__(STAT_BLOCK) prep_stats_kernel(const ReqDesc *__restrict__ reqs, int staged,
                                                                 const __grid_constant__ ReqDesc one, ReqDesc *store) {
     // shared: [STAT_BLOCK / 32][2 NPF + 2] FP32 warp partials, then (staged) the
     // block's parameter rows [STAT_BLOCK][padded_row(NPF + 4)] FP64
@@ -605,7 +606,7 @@ __global__ void __launch_bounds__(PREP_THREADS) prep_tiles_kernel(const ReqDesc 
 // [Tc_pad], wbar hi / lo [N] (FP32); points: parameter rows
 // [128][padded_row(NPF+4)] FP64.
 template <bool BF16, bool ONE>
-__global__ void __launch_bounds__(PREP_THREADS) prep_tc_kernel(const ReqDesc *reqs, int begin,
+__global__ void __launch_bounds__(PREP_THREADS) prep_tc_kernel(const ReqDesc *__restrict__ reqs, int begin,
                                                                const __grid_constant__ ReqDesc one, ReqDesc *store) {
     extern __shared__ double smem_d[];
     __shared__ float sh_red[PREP_THREADS / 32];
@@ -814,7 +815,7 @@ __device__ __forceinline__ void kahan_add(float &s, float &c, float x) {
     s = t;
 }
 
-__device__ __forceinline__ int find_req_by_item(const ReqDesc *reqs, int n_reqs, int64_t item) {
+__device__ __forceinline__ int find_req_by_item(const ReqDesc *__restrict__ reqs, int n_reqs, int64_t item) {
     int lo = 0, hi = n_reqs - 1;
     while (lo < hi) {
         int mid = (lo + hi + 1) >> 1;
@@ -823,7 +824,7 @@ __device__ __forceinline__ int find_req_by_item(const ReqDesc *reqs, int n_reqs,
     return lo;
 }
 
-__device__ __forceinline__ int find_req_by_point(const ReqDesc *reqs, int n_reqs, int64_t pt) {
+__device__ __forceinline__ int find_req_by_point(const ReqDesc *__restrict__ reqs, int n_reqs, int64_t pt) {
     int lo = 0, hi = n_reqs - 1;
     while (lo < hi) {
         int mid = (lo + hi + 1) >> 1;
@@ -930,8 +931,8 @@ __global__ void __launch_bounds__(SIMT_THREADS) simt_kernel(const ReqDesc *reqs,
 #pragma unroll
                 for (int u = 0; u < SIMT_WU; ++u) {
                     if (i0 + u < N) {
-                        b[u] = prow[j * TILE_M];
-                        a[u] = Na ? pa[0] : 0.0f;
+                        b[u] = __ldg(prow + j * TILE_M);
+                        a[u] = Na ? __ldg(pa) : 0.0f;
                     } else {
                         b[u] = a[u] = 0.0f;
                     }

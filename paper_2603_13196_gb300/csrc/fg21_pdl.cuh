@@ -11,12 +11,17 @@
 // dependents' blocks then sit on the SMs beside the running kernel and cost
 // more than the overlap gains.
 //
-// What the earlier kernels of the chain write (a call's only descriptor among
-// it) is read by plain loads, after the wait.  Neither __restrict__ on a kernel's
-// pointer to it nor __ldg may be used: both declare the memory unchanging while
-// the kernel runs, which it is not (the kernel may be resident before the one
-// that writes it has finished), and the compiler may then move a load whose
-// address it knows to before the wait.
+// What the earlier kernels of the chain write must not be read before the wait.
+// __restrict__ on a kernel's pointer and __ldg let the compiler move a load whose
+// address it knows to before it, so:
+//  - a kernel that reads a descriptor which the call's first kernel may have stored
+//    has no __restrict__ on that parameter (a function called after the wait may);
+//  - __ldg is for addresses that were themselves read after the wait, by a plain
+//    load: not in a kernel whose descriptor is an argument by value.
+// (As no kernel triggers its dependents early, every block that writes has ended
+// when a reader's first block starts.)  With plain loads in the tensor kernel
+// instead of __ldg: 64 points, 3 regions 17.8 us a call for 16.7, near the posterior
+// (16384 points) 110.6 for 110.1; with __restrict__ nowhere: 32 models 498 for 494.
 #pragma once
 #include <cuda_runtime.h>
 #include <utility>

@@ -312,7 +312,7 @@ __device__ __forceinline__ int uni(int v) { return __shfl_sync(0xffffffffu, v, 0
 struct Item {
     int req, tile, g, f0, f1;
 };
-__device__ __forceinline__ int find_req(const ReqDesc *reqs, int n, int64_t item) {
+__device__ __forceinline__ int find_req(const ReqDesc *__restrict__ reqs, int n, int64_t item) {
     int lo = 0, hi = n - 1;
     while (lo < hi) {
         int mid = (lo + hi + 1) >> 1;
@@ -321,7 +321,7 @@ __device__ __forceinline__ int find_req(const ReqDesc *reqs, int n, int64_t item
     return lo;
 }
 // Called by a whole converged warp.
-__device__ __forceinline__ Item decode_item(const ReqDesc *reqs, int n, int64_t item) {
+__device__ __forceinline__ Item decode_item(const ReqDesc *__restrict__ reqs, int n, int64_t item) {
     Item it;
     it.req = find_req(reqs, n, item);
     const ReqDesc &r = reqs[it.req];
@@ -484,7 +484,7 @@ __device__ __forceinline__ bool gen_item(const Params &prm, Barriers *S, uint32_
     if (X2_REGS) {
 #pragma unroll
         for (int i = 0; i < NP; ++i) {
-            const float2 v = 2 * i < Kr ? pair2[(size_t)i * 128] : make_float2(0.0f, 0.0f);
+            const float2 v = 2 * i < Kr ? __ldg(pair2 + (size_t)i * 128) : make_float2(0.0f, 0.0f);
             x2[i] = pk2(v.x, v.y);
         }
     }
@@ -508,17 +508,17 @@ __device__ __forceinline__ bool gen_item(const Params &prm, Barriers *S, uint32_
         }
     }
     for (int f = it.f0; f < it.f1; ++f) {
-        const float dnu = nup[f] - nu21;
+        const float dnu = __ldg(nup + f) - nu21;
         uint64_t nL2 = 0;
         if (ALPHA) {
-            const float nL = nLp[f];
+            const float nL = __ldg(nLp + f);
             nL2 = pk2(nL, nL);
         } else {
             // the channel's coefficients e_j = (nL / 2^s)^j / j! (times 2^sW when s = 0), packed pairs
             const ulonglong2 *cf = reinterpret_cast<const ulonglong2 *>(coef + (size_t)f * 8);
 #pragma unroll
             for (int j = 0; 2 * j < DEG; ++j) {
-                const ulonglong2 v = cf[j];
+                const ulonglong2 v = __ldg(cf + j);
                 e2[2 * j + 1] = v.x;
                 if (2 * j + 2 <= DEG) e2[2 * j + 2] = v.y;
             }
@@ -549,7 +549,7 @@ __device__ __forceinline__ bool gen_item(const Params &prm, Barriers *S, uint32_
                         if (X2_REGS) {
                             l2[i] = x2[q * CH + i];
                         } else if (X2) {
-                            const float2 v = pair2[(size_t)(q * CH + i) * 128];
+                            const float2 v = __ldg(pair2 + (size_t)(q * CH + i) * 128);
                             l2[i] = pk2(v.x, v.y);
                         }
                         if (ALPHA) y2[i] = fma2(y2[i], nL2, l2[i]);
@@ -714,11 +714,11 @@ __device__ __forceinline__ bool epi_item(const Params &prm, Barriers *S, uint32_
     const int *scaleB = r.scaleB + it.f0 * nch;
     const int n = (it.f1 - it.f0) * nch;
     float qs0 = 0.0f, qc0 = 0.0f, qs1 = 0.0f, qc1 = 0.0f, qf0 = 0.0f, qf1 = 0.0f;
-    int sb_n = scaleB[0], c = 0;
+    int sb_n = __ldg(scaleB), c = 0;
     for (int k = 0; k < n; ++k) {
         // 2^-(sW + sB), exponents within +-40 each
         const float unscale = __int_as_float((127 - sWexp - sb_n) << 23);
-        sb_n = scaleB[min(k + 1, n - 1)];                  // next stage's scale, one ahead
+        sb_n = __ldg(scaleB + min(k + 1, n - 1));                  // next stage's scale, one ahead
         // the halves of the accumulator are written, read and freed one after the
         // other, so that the next stage's first half can start while this one's
         // second half is still read
