@@ -185,8 +185,8 @@ static int choose_channels_per_group(int64_t total_tiles, int F, int slots, int 
 // channels, 3 to 45 regions and 1 to 100 bins the split taken is the fastest of 13 to
 // within 0.1 us a replay, but for 128 points, 24 regions, 301 channels, 100 bins
 // (1 channel an item 26.7 us, 2 to 6 24.6) and 400 points, 3 regions, one bin (22.6,
-// 21.4 with 3).  Measured against counting waves of single items (16384 points, 301 channels: the same split):
-// 3001 points, 211 channels, two chunks 71 us a call from 78; 8192 points, 301
+// 21.4 with 3).  Measured against counting waves of single items (16384 points, 301
+// channels: the same split): 3001 points, 211 channels, two chunks 71 us a call from 78; 8192 points, 301
 // channels, amplitude regions 91 from 97; 4096 points, 151 channels 29.9 from 31.
 static int choose_channels_tc(int64_t tiles, int F, int n_tchunks, int num_sms) {
     if (g_cpg_override() > 0) return std::min(F, g_cpg_override());
@@ -565,9 +565,8 @@ static int run_host(fg21_model *m, const double *params, int64_t P, double *logL
     m->last_cpg = cpg;
     if (!m->ws.timing && (kept || repeat)) {
         // repeated calls of one size replay a graph of the kernels on the staging
-        // buffers, captured when a size, precision and
-        // tuned work split come twice in a row (a size that changes every call
-        // never pays for a capture)
+        // buffers, captured when a size, precision and tuned work split come twice in
+        // a row (a size that changes every call never pays for a capture)
         if (!kept) {
             if (m->host_graph) {
                 fg21_graph_destroy(m->host_graph);
